@@ -125,10 +125,8 @@ enum {
  *               steps (and then synchronises) and fails with LBM_EUNSTABLE
  *               on a non-finite value or |u| > 0.4
  *  flags        LBM_FLAG_NO_TMA: step with the register-pipelined kernel
- *               instead of the TMA-staged ones (Allen-Cahn and
- *               Cahn-Hilliard; same arithmetic, for A/B comparison);
- *               0 otherwise.  Grids under 16 columns always use the
- *               register-pipelined kernel.
+ *               instead of the tile and TMA-staged ones (Allen-Cahn and
+ *               Cahn-Hilliard; for A/B comparison); 0 otherwise.
  *  n_delta      regularisation of the interface normal of Eq. (8),
  *               n = grad phi / (|grad phi|^4 + delta^4)^(1/4) with
  *               delta = n_delta (phiA - phiB) / W (the paper's grad phi /
@@ -260,11 +258,14 @@ int lbm_set_fields(lbm_handle *h, int32_t which, const double *in);
  * diagnostics sum over fluid nodes and average over fluid nodes without a
  * reflecting link.
  * Takes effect from the next call; call it before lbm_init_fields so that
- * the initial state holds no populations at solid nodes.  With obstacles a
- * step first forms phi (Cahn-Hilliard: and mu_phi) on a whole plane and
- * fills it at the solid nodes next to fluid, then runs the TMA step kernel
- * reading those planes (3 launches a step; 5 for Cahn-Hilliard; with
- * LBM_FLAG_NO_TMA or under 16 columns a one-thread-per-node update instead).
+ * the initial state holds no populations at solid nodes.  With obstacles an
+ * FP32 or FP64 Allen-Cahn step stays one launch, whose blocks near an
+ * obstacle form phi and its fill themselves.  A 16-bit or Cahn-Hilliard step
+ * first forms phi (Cahn-Hilliard: and mu_phi) on a plane, filled at the solid
+ * nodes next to fluid, around the obstacle, then runs the TMA step kernel
+ * reading those planes (2 launches a step; 4 for Cahn-Hilliard).  With
+ * LBM_FLAG_NO_TMA or under 16 columns a one-thread-per-node update over whole
+ * planes runs instead.
  * Device memory: a 2-byte link word per node, two work planes of the
  * arithmetic type and the list of solid nodes next to fluid.  The adjoint
  * entry points return LBM_EUNSUPPORTED while obstacles are set.

@@ -19,6 +19,8 @@
 
 using namespace pflbm;
 
+static constexpr double N_DELTA_DEFAULT = 5e-3;  // lbm_params.n_delta == 0
+
 struct lbm_handle {
   lbm_params prm;
   cudaStream_t stream = nullptr;
@@ -234,7 +236,11 @@ static Phys<T> make_phys(const lbm_handle* h) {
   P.beta4 = T(4.0 * h->beta);
   P.kappa = T(h->kappa);
   P.lam_coef = T(h->lam_coef);
-  P.n_delta = T((Q.n_delta > 0.0 ? Q.n_delta : 5e-3) * (Q.phiA - Q.phiB) / Q.width);
+  P.n_delta = T((Q.n_delta > 0.0 ? Q.n_delta : N_DELTA_DEFAULT) * (Q.phiA - Q.phiB) / Q.width);
+  // its 4th power in T; in FP64 kept above the subnormals (the reciprocal
+  // root's hardware seed flushes them), where it regularises nothing
+  P.n_delta4 = (P.n_delta * P.n_delta) * (P.n_delta * P.n_delta);
+  if (sizeof(T) == 8) P.n_delta4 = std::max(P.n_delta4, T(1e-290));
   P.drho = T(h->drho);
   P.rhoB = T(Q.rhoB);
   P.rho_mean = T(0.5 * (Q.rhoA + Q.rhoB));
@@ -262,6 +268,27 @@ static Phys<T> make_phys(const lbm_handle* h) {
     P.dv_is[set] = T(1.0 / h->dv_s[set]);
   }
   P.dv_c0 = T(h->dv_c0);
+  P.c_eta9 = T(Q.eta / 9.0);
+  P.c_ugq = T((0.5 + h->H) * h->drho);
+  P.c_ug7 = T(2.0 / 3.0 * h->drho);
+  P.c_ug8 = T(1.0 / 3.0 * h->drho);
+  P.c_ug24 = T(-h->drho / 24.0);
+  {
+    // Eq. (11): rho / (3 mu + rho / 2); Eq. (12): (1/nu) / (3 + (1/nu) / 2)
+    const double idp = 1.0 / (Q.phiA - Q.phiB);
+    if (Q.visc_law == LBM_INVERSE_NU) {
+      const double b0 = Q.rhoB / Q.muB, b1 = (Q.rhoA / Q.muA - b0) * idp;
+      P.c_num1 = T(b1), P.c_num0 = T(b0), P.c_den1 = T(0.5 * b1), P.c_den0 = T(3.0 + 0.5 * b0);
+    } else {
+      P.c_num1 = T(h->drho), P.c_num0 = T(Q.rhoB);
+      P.c_den1 = T(3.0 * (Q.muA - Q.muB) * idp + 0.5 * h->drho), P.c_den0 = T(3.0 * Q.muB + 0.5 * Q.rhoB);
+    }
+  }
+  for (int c = 0; c < 2; ++c) {
+    const double sj = h->sf[3 + 2 * c], sq = h->sg[4 + 2 * c];
+    P.c_fa[c][0] = T((1.0 - sj) / 6.0), P.c_fa[c][1] = T(sj / 6.0), P.c_fa[c][2] = T((1.0 - 0.5 * sj) / 6.0);
+    P.c_gn[c][0] = T(-sq / 12.0), P.c_gn[c][1] = T((1.0 - sq) / 12.0), P.c_gn[c][2] = T(-(1.0 - 0.5 * sq) / 12.0);
+  }
   P.obs = h->dobs;
   P.obs_fill = h->dfill;
   P.obs_nfill = h->nfill;
@@ -317,12 +344,23 @@ static int check_device_flag(lbm_handle* h) {
   return LBM_OK;
 }
 
+// Whether the handle's passes run one node per thread (k_tile): plain storage,
+// no obstacles.  LBM_FLAG_NO_TMA asks for the register-pipelined kernel.
+template <class C>
+static bool use_tile(const lbm_handle* h) {
+  return !C::dev && h->use_tma && !h->dobs;
+}
+
 // One pass of the fused kernel in a mode, or, with solid obstacles, the
 // obstacle passes (pflbm_obstacle.cuh).
 template <class C>
 static cudaError_t launch_mode(lbm_handle* h, int mode, const Phys<typename C::value_t>& P,
                                const Bufs<typename C::value_t>& B) {
   using T = typename C::value_t;
+  if constexpr (!C::dev)
+    if (use_tile<C>(h))
+      return launch_tile<C>(h->prm.phase_model, mode, P, B, h->unit_rates,
+                            h->prm.n_delta > 0.0 && h->prm.n_delta < N_DELTA_DEFAULT, h->stream);
   if (!h->dobs) return launch_march<C>(h->prm.phase_model, mode, P, B, h->stream);
   T* phis = (T*)h->obs_planes;
   return launch_obs<C>(h->prm.phase_model, mode, P, B, phis, phis + h->plane, h->unit_rates, h->derr, h->use_tma,
@@ -379,12 +417,13 @@ static int do_step(lbm_handle* h, int64_t n) {
     Bufs<T> B = bufs_now<T>(h);
     B.phi_prev = record ? (T*)h->phi_prev : nullptr;
     cudaError_t e = cudaErrorNotSupported;
-    if (h->dobs)
+    if (h->dobs || use_tile<C>(h)) {
       e = launch_mode<C>(h, MODE_STEP, P, B);
-    else if (h->use_tma && h->prm.phase_model == LBM_AC)
-      e = launch_step_tma<C>(P, B, h->derr, h->unit_rates, h->stream);
-    else if (h->use_tma && h->prm.phase_model == LBM_CH)
-      e = launch_step_tma_ch<C>(P, B, h->derr, h->unit_rates, h->stream);
+    } else if constexpr (C::dev) {
+      if (h->use_tma)
+        e = h->prm.phase_model == LBM_CH ? launch_step_tma_ch<C>(P, B, h->derr, h->unit_rates, h->stream)
+                                         : launch_step_tma<C>(P, B, h->derr, h->unit_rates, h->stream);
+    }
     if (e == cudaErrorNotSupported) e = launch_march<C>(h->prm.phase_model, MODE_STEP, P, B, h->stream);
     CUDA_TRY(h, e);
     h->cur ^= 1;
@@ -609,8 +648,7 @@ static int do_set_fields(lbm_handle* h, int which, const double* in) {
 template <class C>
 static int build_near_map(lbm_handle* h, const uint8_t* solid, bool ch) {
   int tbx = 0, seg = 0;
-  if (ch) tma_ch_step_grid<C>(h->nx, h->ny, &tbx, &seg);
-  else tma_step_grid<C>(h->nx, h->ny, &tbx, &seg);
+  obs_step_grid<C>(h->nx, h->ny, ch, &tbx, &seg);
   const int nx = h->nx, ny = h->ny;
   const bool px = h->prm.bc[LBM_LEFT] == LBM_PERIODIC, py = h->prm.bc[LBM_BOTTOM] == LBM_PERIODIC;
   const int gx = (nx + tbx - 1) / tbx, gy = (ny + seg - 1) / seg;

@@ -2,8 +2,10 @@
 //
 // Method: Zhan, Chai & Shi, "Consistent and conservative phase-field based
 // lattice Boltzmann method for incompressible two-phase flows"
-// (arXiv:2111.00847), Sec. 3 and App. C.  One launch of k_march<T, MODEL,
-// MODE_STEP> advances the whole grid by one time step.
+// (arXiv:2111.00847), Sec. 3 and App. C.  One launch of a step kernel advances
+// the whole grid by one time step: k_tile (FP32 and FP64 storage), k_step_tma
+// and k_step_tma_ch (16-bit storage; Cahn-Hilliard with obstacles), or k_march
+// (on request).
 //
 // Memory layout (HBM).  Populations are structure-of-arrays planes, one per
 // D2Q9 direction, interleaved by rows: element i of node (x, y) of a set of
@@ -77,7 +79,7 @@ struct Phys {
   int gravity_mode, visc_inverse, sg7_node, sg8_node;
   T phiA, phiB, phibar, inv_dphi;
   T beta4, kappa, lam_coef;  // 4 beta, k, sqrt(2 beta / k)   (Eqs. (3), (5), (8))
-  T n_delta;                 // regularisation of |grad phi| in n = grad phi / |grad phi|
+  T n_delta, n_delta4;       // regularisation of |grad phi| in n = grad phi / |grad phi|, and its 4th power
   T drho, rhoB, rho_mean;    // d rho / d phi, rho_B, (rho_A + rho_B)/2
   T mob_drho;                // (d rho/d phi) M_phi, zero for the original model
   T muA, muB, inuA, inuB;    // mu_A, mu_B, 1/nu_A, 1/nu_B
@@ -90,6 +92,15 @@ struct Phys {
   // scale s of the stored deviations and 1/s, and for f the factor
   // 1 / (1 + sum_i r_i) that makes a node's decoded populations sum to phi.
   T dv_r[2][2], dv_s[2], dv_is[2], dv_c0;
+  // FP64 node update: combinations of the constants above, so that no thread
+  // forms them again (see node_update)
+  T c_eta9;                  // eta / 9
+  T c_ugq, c_ug7, c_ug8;     // (1/2 + H) drho, 2/3 drho, 1/3 drho
+  T c_ug24;                  // -drho / 24
+  T c_num1, c_num0;          // viscous rate = num / den, num = num1 (phi - phi_B) + num0, den likewise
+  T c_den1, c_den0;
+  T c_fa[2][3];              // f, moments (3, 4) and (5, 6): j/6 relaxed = fa . (m, phi u, X)
+  T c_gn[2][3];              // g, moments 4 and 6: relaxed q/12 = gn . (rho u, m, F)
   int seg_rows;  // rows per block segment of the TMA step on small grids (set by its launcher)
   int diag_y0, diag_y1;  // rows [diag_y0, diag_y1) enter the diagnostics (a y-slab: its own rows)
   // Solid obstacles (nullptr: none).  Per node of the dense [ny][nx] grid:
@@ -362,6 +373,30 @@ __device__ __forceinline__ void store_pops(const Phys<typename C::value_t>& P, v
   }
 }
 
+// Where a node update puts its outputs.  NodeSink addresses node (x, y) of the
+// planes; INIT writes plain values, the other modes the codec's.
+template <class C, int MODE, typename T = typename C::value_t>
+struct NodeSink {
+  using CS = typename std::conditional<MODE == MODE_INIT, PopPlain<T>, C>::type;
+  const Phys<T>& P;
+  const Bufs<T>& B;
+  int x, y;
+  __device__ __forceinline__ void hist(T a, T b, T c, T d, T e, T phi) const {
+    const long long pc = P.pitch;
+    T* hb = B.hist + ix(P, 5, 0, x, y);
+    hb[0] = a;
+    hb[pc] = b;
+    hb[2 * pc] = c;
+    hb[3 * pc] = d;
+    hb[4 * pc] = e;
+    if (B.phi_prev) B.phi_prev[ix(P, 1, 0, x, y)] = phi;
+  }
+  __device__ __forceinline__ T* macro() const { return B.macro + ix(P, NMACRO, 0, x, y); }
+  __device__ __forceinline__ void pops(int set, const T v[9], T m0, bool conserve) const {
+    store_pops<CS>(P, set ? B.gout : B.fout, set, x, y, v, m0, conserve);
+  }
+};
+
 template <typename T>
 __device__ __forceinline__ T sum9(const T v[9]) {
   return ((v[0] + (v[1] + v[3])) + (v[2] + v[4])) + ((v[5] + v[7]) + (v[6] + v[8]));
@@ -406,18 +441,393 @@ __device__ __forceinline__ T wall_ghost(const Phys<T>& P, int side, T phi1, T ph
 }
 
 // ---------------------------------------------------------------------------
-// Per-node update.  phi9 / mu9: values at x + c_i (D2Q9 order), f, g: pulled
-// populations, h: chi(t-1).  Writes the outputs of the mode.
+// FP64 arithmetic of the node update.  GB300's FP64 pipe (two instructions a
+// clock and SM) bounds every FP64 kernel here, so operations are counted, and
+// each is written out with its own rounding (the compiler contracts nothing):
+// all kernels that update a node return the same bits, whichever of them the
+// size of a grid (or of a y-slab of it) selects.
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ double fm(double a, double b, double c) { return __fma_rn(a, b, c); }
+__device__ __forceinline__ double ad(double a, double b) { return __dadd_rn(a, b); }
+__device__ __forceinline__ double sb(double a, double b) { return __dsub_rn(a, b); }
+__device__ __forceinline__ double ml(double a, double b) { return __dmul_rn(a, b); }
+
+// 1 / a: the hardware's seed (rcp.approx.ftz.f64; its relative error was
+// measured below 2^-19.9) and one step of the third-order iteration
+// y (1 + e + e^2), e = 1 - a y (the geometric series of 1 / (1 - e); the
+// remainder e^3 is below 2^-59).  Three FP64 operations where an IEEE division
+// takes about nine; measured largest error 2^-53.0, as correct rounding.
+__device__ __forceinline__ double recip(double a) {
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(a));
+  const double e = fm(-a, y, 1.0);
+  return fm(y, fm(e, e, e), y);
+}
+// S^(-1/4): z = y y^(-1/2) with y = S^(-1/2), both from the hardware's seed
+// (rsqrt.approx.ftz.f64; z was measured good to 2^-19.7), then
+// z (1 + e/4 + 5/32 e^2), e = 1 - S z^4, the binomial series of
+// (1 - e)^(-1/4).  Seven operations; measured largest error 2^-52.3 (2^-52.0
+// for 1 / sqrt(sqrt(S)), which takes about thirty).
+__device__ __forceinline__ double inv_root4(double S) {
+  double r, q;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(S));
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(q) : "d"(r));
+  const double z = ml(r, q), z2 = ml(z, z);
+  const double e = fm(-ml(S, z2), z2, 1.0);
+  return fm(z, ml(e, fm(5.0 / 32, e, 0.25)), z);
+}
+
+// A field on one row of a node's 3 x 3 stencil: its value c in the node's
+// column, h = right - left and q = right - 2 c + left (from differences, which
+// are exact for neighbouring values).  The isotropic stencils of Eqs.
+// (C.9)-(C.10) are sums of these over the rows below, at and above the node,
+//   grad_x = h_0 / 3 + (h_+ + h_-) / 12,
+//   grad_y = (c_+ - c_-) / 2 + (q_+ - q_-) / 12,
+//   lap    = (c_+ - c_0) + (c_- - c_0) + 2/3 q_0 + (q_+ + q_-) / 6,
+// 17 operations with h and q of one new row per node, against 26 from the
+// nine values; a marching kernel keeps the two older rows in registers and
+// reads three values per row instead of nine.
+template <typename T>
+struct Row3 {
+  T c, h, q;
+};
+template <typename T>
+__device__ __forceinline__ Row3<T> row3(T l, T c, T r) {
+  return Row3<T>{c, sb(r, l), ad(sb(r, c), sb(l, c))};
+}
+template <typename T>
+__device__ __forceinline__ Row3<T> row3_at(const T* c) {
+  return row3(c[-1], c[0], c[1]);
+}
+template <typename T>
+__device__ __forceinline__ T grad_x(const Row3<T>& m, const Row3<T>& o, const Row3<T>& p) {
+  return fm(T(1.0 / 12.0), ad(p.h, m.h), ml(T(1.0 / 3.0), o.h));
+}
+template <typename T>
+__device__ __forceinline__ T grad_y(const Row3<T>& m, const Row3<T>& p) {
+  return fm(T(1.0 / 12.0), sb(p.q, m.q), ml(T(0.5), sb(p.c, m.c)));
+}
+template <typename T>
+__device__ __forceinline__ T laplace(const Row3<T>& m, const Row3<T>& o, const Row3<T>& p) {
+  const T v = ad(sb(p.c, o.c), sb(m.c, o.c));
+  return fm(T(1.0 / 6.0), ad(p.q, m.q), fm(T(2.0 / 3.0), o.q, v));
+}
+// chemical potential, Eq. (5)
+template <typename T>
+__device__ __forceinline__ T chem_pot(const Phys<T>& P, const Row3<T>& m, const Row3<T>& o, const Row3<T>& p) {
+  const T phi = o.c;
+  const T pab = ml(sb(phi, P.phiA), sb(phi, P.phiB));
+  return fm(ml(P.beta4, sb(phi, P.phibar)), pab, ml(-P.kappa, laplace(m, o, p)));
+}
+
+// nine values in D2Q9 order as rows
+template <typename T>
+__device__ __forceinline__ void rows_of(const T v[9], Row3<T> r[3]) {
+  r[0] = row3(v[7], v[4], v[8]);
+  r[1] = row3(v[3], v[0], v[1]);
+  r[2] = row3(v[6], v[2], v[5]);
+}
+
+// M^{-1} m (the basis of Eq. (C.1), orthogonal rows) for the populations of
+// a set: m_0, m_1, m_2 are given combined into v0 (rest), a (axis) and b
+// (diagonal directions), the vector moments as j = m_{3,5}/6 and
+// r = m_{4,6}/12, which enter the axes as j - 2 r and the diagonals as j + r.
+template <typename T>
+__device__ __forceinline__ void populate(T v0, T ap, T am, T bp, T bm, T jx, T rx, T jy, T ry, T out[9]) {
+  const T X = fm(T(-2), rx, jx), Y = fm(T(-2), ry, jy);
+  const T Xd = ad(jx, rx), Yd = ad(jy, ry);
+  const T S = ad(Xd, Yd), D = sb(Xd, Yd);
+  out[0] = v0;
+  out[1] = ad(ap, X);
+  out[3] = sb(ap, X);
+  out[2] = ad(am, Y);
+  out[4] = sb(am, Y);
+  out[5] = ad(bp, S);
+  out[7] = sb(bp, S);
+  out[8] = ad(bm, D);
+  out[6] = sb(bm, D);
+}
+// the same with the moments 7 and 8
+template <typename T>
+__device__ __forceinline__ void populate78(T v0, T a, T b, T jx, T rx, T jy, T ry, T m7, T m8, T out[9]) {
+  populate(v0, fm(T(0.25), m7, a), fm(T(-0.25), m7, a), fm(T(0.25), m8, b), fm(T(-0.25), m8, b), jx, rx, jy, ry, out);
+}
+
+// Sums and differences of a set's populations over opposite directions, from
+// which all nine moments M v follow.
+template <typename T>
+struct Pairs {
+  T s13, s24, s57, s68, d13, d24, gx, gy;  // gx, gy: the diagonals' x and y differences
+};
+template <typename T>
+__device__ __forceinline__ Pairs<T> pairs_of(const T v[9]) {
+  Pairs<T> o;
+  o.s13 = ad(v[1], v[3]);
+  o.s24 = ad(v[2], v[4]);
+  o.s57 = ad(v[5], v[7]);
+  o.s68 = ad(v[6], v[8]);
+  o.d13 = sb(v[1], v[3]);
+  o.d24 = sb(v[2], v[4]);
+  const T d57 = sb(v[5], v[7]), d86 = sb(v[8], v[6]);
+  o.gx = ad(d57, d86);
+  o.gy = sb(d57, d86);
+  return o;
+}
+// general relaxation (UR = false): m <- M v relaxed at s towards eq with the
+// source src, then the populations
+template <typename T>
+__device__ __forceinline__ void relax_general(const T v[9], const Pairs<T>& o, const T eq[9], const T src[9],
+                                              const T s[9], const T hs[9], T out[9]) {
+  const T sa = ad(o.s13, o.s24), sd = ad(o.s57, o.s68);
+  T m[9];
+  m[0] = ad(ad(v[0], sa), sd);
+  m[1] = fm(T(-4), v[0], fm(T(2), sd, -sa));
+  m[2] = fm(T(4), v[0], fm(T(-2), sa, sd));
+  m[3] = ad(o.d13, o.gx);
+  m[4] = fm(T(-2), o.d13, o.gx);
+  m[5] = ad(o.d24, o.gy);
+  m[6] = fm(T(-2), o.d24, o.gy);
+  m[7] = sb(o.s13, o.s24);
+  m[8] = sb(o.s57, o.s68);
+#pragma unroll
+  for (int k = 0; k < 9; ++k) m[k] = fm(hs[k], src[k], fm(s[k], sb(eq[k], m[k]), m[k]));
+  const T n0 = ml(T(1.0 / 9.0), m[0]);
+  const T a = fm(T(-1.0 / 18.0), m[2], fm(T(-1.0 / 36.0), m[1], n0));
+  const T b = fm(T(1.0 / 36.0), m[2], fm(T(1.0 / 18.0), m[1], n0));
+  populate78(ml(T(1.0 / 9.0), ad(sb(m[0], m[1]), m[2])), a, b, ml(T(1.0 / 6.0), m[3]), ml(T(1.0 / 12.0), m[4]),
+             ml(T(1.0 / 6.0), m[5]), ml(T(1.0 / 12.0), m[6]), m[7], m[8], out);
+}
+
+// ---------------------------------------------------------------------------
+// Per-node update in FP64.  fr, mr: phi (Cahn-Hilliard: and mu_phi) on the rows below,
+// at and above the node; f, g: pulled populations; h: chi(t-1).  Writes the
+// outputs of the mode.
 // ---------------------------------------------------------------------------
 // UR ("unit rates"): the relaxation rates of Sec. 4 that the paper leaves at
 // 1 are 1 (s_f^k for k != 3, 5 and s_g^k for k = 0, 1, 2, 3, 5); those
 // moments then relax to m^eq + m_src / 2 without reading the populations'
-// own moments, which the general path (UR = false) computes and relaxes.
+// own moments, and the even ones are put straight into the populations they
+// enter, with the constants of Eqs. (C.2)-(C.4) and M^{-1} multiplied out:
+//   f: f_0 = phi - 5/9 eta chi, axis eta chi / 9, diagonal eta chi / 36
+//      (chi = phi for Allen-Cahn, mu_phi for Cahn-Hilliard), which sum to phi;
+//   g: with q = p / 0.6, Z = rho u.u + u.m, w = Z + (d_t(u.m) + 2 u.F) / 2 and
+//      r = u.grad rho: g_0 = -q - 2/3 w, axis q/5 + (w + r)/12,
+//      diagonal q/20 + (w + r)/12 - r/24.
+// rho u is Eq. (22b)'s numerator, and m^{phi C} is parallel to grad phi
+// (Allen-Cahn), so its products with u are multiples of u's with grad phi.
+// The general path (UR = false) computes and relaxes all nine moments.
 // C: the storage codec of the STEP outputs (INIT writes plain values).
-template <class C, int MODEL, int MODE, bool UR = false, typename T = typename C::value_t>
-__device__ __forceinline__ void node_update(const Phys<T>& P, const Bufs<T>& B, int x, int y,
-                                            const T phi9[9], const T mu9[9], const T f[9],
-                                            const T g[9], const T h[5], T u_in, T v_in, T p_in) {
+template <class C, int MODEL, int MODE, bool UR, class Sink, typename T = typename C::value_t>
+__device__ __forceinline__ void node_update(const Phys<T>& P, const Sink& out, const Row3<T> fr[3],
+                                            const Row3<T> mr[3], const T f[9], const T g[9], const T h[5],
+                                            T u_in, T v_in, T p_in) {
+  const T phi = fr[1].c;
+  const long long pc = P.pitch;
+  const T gx = grad_x(fr[0], fr[1], fr[2]), gy = grad_y(fr[0], fr[2]);
+  const T pb = sb(phi, P.phiB);
+  T mu, Dx = T(0), Dy = T(0);
+  T li = T(0);  // Allen-Cahn: -lambda r, with n = r grad phi
+  T cm = T(0);  // Allen-Cahn: m^{phi C} = cm grad phi
+  if (MODEL == MODEL_AC) {
+    mu = chem_pot(P, fr[0], fr[1], fr[2]);
+    // conservative AC flux, Eqs. (7)-(8), D = grad phi - lambda n with
+    // n = grad phi / (|grad phi|^4 + delta_n^4)^(1/4) (delta_n = n_delta dphi / W:
+    // the unit normal across the interface, and a smooth function of grad phi
+    // with slope about 1/delta_n in the bulk, where |grad phi| -> 0)
+    const T g2 = fm(gx, gx, ml(gy, gy));
+    li = ml(ml(P.lam_coef, ml(sb(phi, P.phiA), pb)), inv_root4(fm(g2, g2, P.n_delta4)));
+    cm = fm(-P.mob_drho, li, -P.mob_drho);
+  } else {
+    // CH: D = grad mu_phi (Eq. (6))
+    mu = mr[1].c;
+    Dx = grad_x(mr[0], mr[1], mr[2]);
+    Dy = grad_y(mr[0], mr[2]);
+  }
+  // density (Eq. (10)), force; its gradient is drho grad phi
+  const T rho = fm(P.drho, pb, P.rhoB);
+  const T Gs = P.gravity_mode == 0 ? T(1) : (P.gravity_mode == 1 ? rho : sb(rho, P.rho_mean));
+  const T Fx = fm(mu, gx, ml(Gs, P.gx)), Fy = fm(mu, gy, ml(Gs, P.gy));
+
+  const Pairs<T> pg = pairs_of(g);
+  const T gab = ad(ad(pg.s13, pg.s24), ad(pg.s57, pg.s68));
+  T u, v, E3, E5;  // u and rho u (the moments 3, 5 of g^eq)
+  if (MODE == MODE_INIT) {
+    u = u_in;
+    v = v_in;
+    E3 = ml(rho, u);
+    E5 = ml(rho, v);
+  } else {
+    // Eq. (22b): rho u = sum c_i g_i + F/2
+    const T irho = recip(rho);
+    E3 = fm(T(0.5), Fx, ad(pg.d13, pg.gx));
+    E5 = fm(T(0.5), Fy, ad(pg.d24, pg.gy));
+    u = ml(E3, irho);
+    v = ml(E5, irho);
+  }
+  // products with grad phi: u.grad, u gx - v gy, u gy + v gx
+  const T vgy = ml(v, gy);
+  const T ug = fm(u, gx, vgy), ugm = fm(u, gx, -vgy), ugx = fm(u, gy, ml(v, gx));
+  // with m^{phi C} (Eq. (15)): u.m, u m_x - v m_y, u m_y + v m_x
+  T um, cA, cB, mcx = T(0), mcy = T(0);
+  if (MODEL == MODEL_AC) {
+    um = ml(cm, ug);
+    cA = ml(cm, ugm);
+    cB = ml(cm, ugx);
+    if (MODE == MODE_MACRO) mcx = ml(cm, gx), mcy = ml(cm, gy);
+  } else {
+    mcx = ml(-P.mob_drho, Dx), mcy = ml(-P.mob_drho, Dy);
+    const T vmy = ml(v, mcy);
+    um = fm(u, mcx, vmy), cA = fm(u, mcx, -vmy), cB = fm(u, mcy, ml(v, mcx));
+  }
+  const T phu = ml(phi, u), phv = ml(phi, v);
+  T d_phu = T(0), d_phv = T(0), d_um = T(0), d_A = T(0), d_B = T(0);
+  if (MODE == MODE_STEP || MODE == MODE_MACRO) {
+    d_phu = sb(phu, h[0]);
+    d_phv = sb(phv, h[1]);
+    d_um = sb(um, h[2]);
+    d_A = sb(cA, h[3]);
+    d_B = sb(cB, h[4]);
+  }
+  if (MODE == MODE_HIST || MODE == MODE_STEP) {
+    out.hist(phu, phv, um, cA, cB, phi);
+    if (MODE == MODE_HIST) return;
+  }
+  // products with F, and Z = rho u.u + u.m
+  const T vFy = ml(v, Fy);
+  const T uF = fm(u, Fx, vFy), uFm = fm(u, Fx, -vFy), uFx = fm(u, Fy, ml(v, Fx));
+  const T Z = fm(u, E3, fm(v, E5, um));
+  const T t = fm(T(2), uF, d_um);
+  T q;  // p / 0.6
+  if (MODE == MODE_INIT) {
+    q = ml(T(5.0 / 3.0), p_in);
+  } else {
+    // Eq. (39), second way: s_0 = -w_0 (rho u.u + u.m)/(2 c_s^2) = -(2/3) Z
+    q = fm(P.K, t, fm(T(-2.0 / 3.0), Z, fm(P.c_ugq, ug, gab)));
+  }
+
+  // viscous rate s_g^{7,8} = 1/(nu/c_s^2 + 1/2), nu from Eq. (11) or (12):
+  // a quotient of two linear functions of phi
+  T s7 = P.sg[7], s8 = P.sg[8];
+  if (P.sg7_node | P.sg8_node) {
+    const T num = P.visc_inverse ? fm(P.c_num1, pb, P.c_num0) : rho;
+    const T snode = ml(num, recip(fm(P.c_den1, pb, P.c_den0)));
+    if (P.sg7_node) s7 = snode;
+    if (P.sg8_node) s8 = snode;
+  }
+
+  if (MODE == MODE_MACRO) {
+    // strain-rate trace, Eq. (35): tr S = -s_2/(2 rho c_s^2)[tr sum cc(g - g^eq) + tr M_2F / 2]
+    const T p = ml(T(0.6), q);
+    const T sd = ad(pg.s57, pg.s68), sa = ad(pg.s13, pg.s24);
+    const T m0 = ad(g[0], gab), m1 = fm(T(-4), g[0], fm(T(2), sd, -sa));
+    const T E1 = fm(T(6), p, ml(T(3), Z)), Q1 = ml(T(3), t);
+    const T trneq = (m1 - E1 + T(4) * m0) * T(1.0 / 3.0);
+    const T trM2F = (Q1 + T(4) * (P.drho * ug)) * T(1.0 / 3.0);
+    const T trS = -s7 * T(1.5) / rho * (trneq + T(0.5) * trM2F);
+    T* M = out.macro();
+    M[MAC_PHI * pc] = phi;
+    M[MAC_UX * pc] = u;
+    M[MAC_UY * pc] = v;
+    M[MAC_P * pc] = p;
+    M[MAC_RHO * pc] = rho;
+    M[MAC_MU * pc] = mu;
+    M[MAC_MCX * pc] = mcx;
+    M[MAC_MCY * pc] = mcy;
+    M[MAC_TRS * pc] = trS;
+    return;
+  }
+
+  // ---- phase-field collision, Eq. (17) with Eq. (C.4) (AC) / (C.3) (CH)
+  const T chi = (MODEL == MODEL_AC) ? phi : mu;
+  T fs[9];
+  T Xx = d_phu, Xy = d_phv;  // d_t(phi u) + lambda n / 3
+  if (MODEL == MODEL_AC && MODE == MODE_STEP) {
+    const T l3 = ml(T(-1.0 / 3.0), li);
+    Xx = fm(l3, gx, d_phu);
+    Xy = fm(l3, gy, d_phv);
+  }
+  if (MODE == MODE_INIT || UR) {
+    const T a = ml(P.c_eta9, chi);
+    const T f0 = fm(T(-5), a, phi), b = ml(T(0.25), a);
+    if (MODE == MODE_INIT) {  // f^eq = M^{-1} m^eq
+      populate(f0, a, a, b, b, ml(T(1.0 / 6.0), phu), ml(T(-1.0 / 12.0), phu), ml(T(1.0 / 6.0), phv),
+               ml(T(-1.0 / 12.0), phv), fs);
+    } else {
+      // only j_x, j_y (moments 3, 5) relax at s_f^{3,5}; the others take
+      // m^eq + m_R / 2 (m_R vanishes in moments 0-2, 7, 8)
+      const T d57 = sb(f[5], f[7]), d86 = sb(f[8], f[6]);
+      const T m3 = ad(sb(f[1], f[3]), ad(d57, d86)), m5 = ad(sb(f[2], f[4]), sb(d57, d86));
+      const T jx = fm(P.c_fa[0][2], Xx, fm(P.c_fa[0][1], phu, ml(P.c_fa[0][0], m3)));
+      const T jy = fm(P.c_fa[1][2], Xy, fm(P.c_fa[1][1], phv, ml(P.c_fa[1][0], m5)));
+      populate(f0, a, a, b, b, jx, fm(T(-1.0 / 24.0), Xx, ml(T(-1.0 / 12.0), phu)), jy,
+               fm(T(-1.0 / 24.0), Xy, ml(T(-1.0 / 12.0), phv)), fs);
+    }
+  } else {
+    const T ec = ml(P.eta, chi);
+    const T eq[9] = {phi, fm(T(-4), phi, ml(T(2), ec)), fm(T(4), phi, ml(T(-3), ec)), phu, -phu, phv, -phv, T(0), T(0)};
+    const T src[9] = {T(0), T(0), T(0), Xx, -Xx, Xy, -Xy, T(0), T(0)};
+    relax_general(f, pairs_of(f), eq, src, P.sf, P.hf, fs);
+  }
+
+  // ---- hydrodynamic collision, Eq. (40) with Eq. (C.2)
+  const T E7 = fm(u, E3, fm(-v, E5, cA));
+  const T E8 = fm(u, E5, ml(T(0.5), cB));
+  T gs[9];
+  if (MODE == MODE_INIT) {  // g^eq
+    const T z12 = ml(T(1.0 / 12.0), Z);
+    populate78(-fm(T(2.0 / 3.0), Z, q), fm(T(0.2), q, z12), fm(T(0.05), q, z12), ml(T(1.0 / 6.0), E3),
+               ml(T(-1.0 / 12.0), E3), ml(T(1.0 / 6.0), E5), ml(T(-1.0 / 12.0), E5), E7, E8, gs);
+  } else {
+    // forcing moments, Eq. (C.2)
+    const T Q7 = fm(P.c_ug7, ugm, fm(T(2), uFm, d_A));
+    const T Q8 = fm(P.c_ug8, ugx, fm(T(0.5), d_B, uFx));
+    if (UR) {
+      const T w = fm(T(0.5), t, Z);
+      const T x12 = ml(T(1.0 / 12.0), fm(P.drho, ug, w));
+      const T a = fm(T(0.2), q, x12);
+      const T b = fm(T(0.05), q, fm(P.c_ug24, ug, x12));
+      const T m4 = fm(T(-2), pg.d13, pg.gx), m6 = fm(T(-2), pg.d24, pg.gy);
+      const T m7 = sb(pg.s13, pg.s24), m8 = sb(pg.s57, pg.s68);
+      const T rx = fm(P.c_gn[0][2], Fx, fm(P.c_gn[0][0], E3, ml(P.c_gn[0][1], m4)));
+      const T ry = fm(P.c_gn[1][2], Fy, fm(P.c_gn[1][0], E5, ml(P.c_gn[1][1], m6)));
+      const T n7 = fm(s7, fm(T(-0.5), Q7, sb(E7, m7)), ad(m7, Q7));
+      const T n8 = fm(s8, fm(T(-0.5), Q8, sb(E8, m8)), ad(m8, Q8));
+      populate78(-fm(T(2.0 / 3.0), w, q), a, b, fm(T(1.0 / 12.0), Fx, ml(T(1.0 / 6.0), E3)), rx,
+                 fm(T(1.0 / 12.0), Fy, ml(T(1.0 / 6.0), E5)), ry, n7, n8, gs);
+    } else {
+      const T ugr = ml(P.drho, ug);
+      const T Q1 = ml(T(3), t);
+      const T p6 = ml(T(3.6), q), z3 = ml(T(3), Z);
+      const T eq[9] = {T(0), ad(p6, z3), -fm(T(1.5), p6, z3), E3, -E3, E5, -E5, E7, E8};
+      const T src[9] = {ugr, Q1, -ad(ugr, Q1), Fx, -Fx, Fy, -Fy, Q7, Q8};
+      T s[9], hs[9];
+#pragma unroll
+      for (int k = 0; k < 7; ++k) s[k] = P.sg[k], hs[k] = P.hg[k];
+      s[7] = s7, hs[7] = fm(T(-0.5), s7, T(1));
+      s[8] = s8, hs[8] = fm(T(-0.5), s8, T(1));
+      relax_general(g, pg, eq, src, s, hs, gs);
+    }
+  }
+
+  out.pops(0, fs, phi, true);
+  out.pops(1, gs, T(0), false);
+}
+
+// ---------------------------------------------------------------------------
+// Per-node update in FP32 arithmetic, through the moments of App. C (phi9 /
+// mu9: values at x + c_i in D2Q9 order); FP64 uses it in k_march and where
+// n_delta is below its default (see launch_tile_moments).  The FP32 and 16-bit steps wait on
+// memory and shared memory, not on arithmetic: node_update's shorter form ran
+// the FP32 steps at the same speed (4096 x 2048 with an obstacle 5 % slower,
+// the 16-bit step 6 % slower: its kept rows need registers) and its fewer,
+// differently placed roundings moved FP32 results by as much as their own
+// error and the BF16 dam break's front by five cells in 4000 steps.
+// UR: as for node_update.
+// ---------------------------------------------------------------------------
+template <class C, int MODEL, int MODE, bool UR, class Sink, typename T = typename C::value_t>
+__device__ __forceinline__ void node_update_moments(const Phys<T>& P, const Sink& out, const T phi9[9],
+                                                    const T mu9[9], const T f[9], const T g[9], const T h[5],
+                                                    T u_in, T v_in, T p_in) {
   const T phi = phi9[0];
   const long long pc = P.pitch;
   // isotropic gradient and Laplacian, Eqs. (C.9)-(C.10) (c_s^2 = 1/3):
@@ -495,15 +905,7 @@ __device__ __forceinline__ void node_update(const Phys<T>& P, const Bufs<T>& B, 
   }
 
   if (MODE == MODE_HIST || MODE == MODE_STEP) {
-    {
-      T* hb = B.hist + ix(P, 5, 0, x, y);
-      hb[0] = phu;
-      hb[pc] = phv;
-      hb[2 * pc] = um;
-      hb[3 * pc] = cA;
-      hb[4 * pc] = cB;
-    }
-    if (B.phi_prev) B.phi_prev[ix(P, 1, 0, x, y)] = phi;
+    out.hist(phu, phv, um, cA, cB, phi);
     if (MODE == MODE_HIST) return;
   }
 
@@ -545,7 +947,7 @@ __device__ __forceinline__ void node_update(const Phys<T>& P, const Bufs<T>& B, 
     const T trneq = ((m1 - E1) + T(4) * m0) * T(1.0 / 3.0);
     const T trM2F = (Q1 + T(4) * Q0) * T(1.0 / 3.0);
     const T trS = -s7 * T(1.5) / rho * (trneq + T(0.5) * trM2F);
-    T* M = B.macro + ix(P, NMACRO, 0, x, y);
+    T* M = out.macro();
     M[MAC_PHI * pc] = phi;
     M[MAC_UX * pc] = u;
     M[MAC_UY * pc] = v;
@@ -679,10 +1081,68 @@ __device__ __forceinline__ void node_update(const Phys<T>& P, const Bufs<T>& B, 
     gs[7] = b - Xd - Yd + Qq; gs[8] = b + Xd - Yd - Qq;
   }
 
-  using CS = typename std::conditional<MODE == MODE_INIT, PopPlain<T>, C>::type;
-  store_pops<CS>(P, B.fout, 0, x, y, fs, phi, true);
-  store_pops<CS>(P, B.gout, 1, x, y, gs, T(0), false);
+  out.pops(0, fs, phi, true);
+  out.pops(1, gs, T(0), false);
 }
+
+// mu_phi (Eq. (5)) at a node from its phi rows, rounded as the node update
+// that follows rounds it
+template <class C, bool MOM = sizeof(typename C::value_t) == 4, typename T = typename C::value_t>
+__device__ __forceinline__ T chem_pot_rows(const Phys<T>& P, const T* pm, const T* p0, const T* pp) {
+  if constexpr (!MOM) return chem_pot(P, row3_at(pm), row3_at(p0), row3_at(pp));
+  const T ph = p0[0];
+  const T lap = (((p0[1] - ph) + (p0[-1] - ph)) + ((pp[0] - ph) + (pm[0] - ph))) * T(2.0 / 3.0) +
+                (((pp[1] - ph) + (pm[-1] - ph)) + ((pp[-1] - ph) + (pm[1] - ph))) * T(1.0 / 6.0);
+  return P.beta4 * (ph - P.phiA) * (ph - P.phiB) * (ph - P.phibar) - P.kappa * lap;
+}
+
+// The update of the arithmetic type, from nine stencil values in D2Q9 order.
+template <class C, int MODEL, int MODE, bool UR, class Sink, typename T = typename C::value_t>
+__device__ __forceinline__ void node_update_nine(const Phys<T>& P, const Sink& out, const T phi9[9], const T mu9[9],
+                                                 const T f[9], const T g[9], const T h[5], T u_in, T v_in, T p_in) {
+  if constexpr (sizeof(T) == 4) {
+    node_update_moments<C, MODEL, MODE, UR>(P, out, phi9, mu9, f, g, h, u_in, v_in, p_in);
+  } else {
+    Row3<T> fr[3], mr[3];
+    rows_of(phi9, fr);
+    if (MODEL == MODEL_CH) rows_of(mu9, mr);
+    node_update<C, MODEL, MODE, UR>(P, out, fr, mr, f, g, h, u_in, v_in, p_in);
+  }
+}
+
+// A node's stencil values in the form its update takes: three rows (FP64), or
+// the nine values in D2Q9 order (MOM, the moment form: FP32, and FP64 where it
+// is asked for).
+template <class C, int MODEL, bool MOM = sizeof(typename C::value_t) == 4>
+struct Stencil {
+  using T = typename C::value_t;
+  Row3<T> fr[3], mr[3];
+  T phi9[9], mu9[9];
+  static __device__ __forceinline__ void nine(const T* m, const T* o, const T* p, T v[9]) {
+    v[0] = o[0], v[1] = o[1], v[2] = p[0], v[3] = o[-1], v[4] = m[0];
+    v[5] = p[1], v[6] = p[-1], v[7] = m[-1], v[8] = m[1];
+  }
+  // m, o, p: the node's column in the rows below, at and above it
+  __device__ __forceinline__ void phi_rows(const T* m, const T* o, const T* p) {
+    if constexpr (MOM) nine(m, o, p, phi9);
+    else fr[0] = row3_at(m), fr[1] = row3_at(o), fr[2] = row3_at(p);
+  }
+  __device__ __forceinline__ void mu_rows(const T* m, const T* o, const T* p) {
+    if constexpr (MOM) nine(m, o, p, mu9);
+    else mr[0] = row3_at(m), mr[1] = row3_at(o), mr[2] = row3_at(p);
+  }
+  template <int MODE, bool UR, class Sink>
+  __device__ __forceinline__ void update(const Phys<T>& P, const Sink& out, const T f[9], const T g[9],
+                                         const T h[5], T u, T v, T p) {
+    if constexpr (MOM) node_update_moments<C, MODEL, MODE, UR>(P, out, phi9, mu9, f, g, h, u, v, p);
+    else node_update<C, MODEL, MODE, UR>(P, out, fr, mr, f, g, h, u, v, p);
+  }
+  template <int MODE, bool UR>
+  __device__ __forceinline__ void update(const Phys<T>& P, const Bufs<T>& B, int x, int y, const T f[9],
+                                         const T g[9], const T h[5], T u, T v, T p) {
+    update<MODE, UR>(P, NodeSink<C, MODE>{P, B, x, y}, f, g, h, u, v, p);
+  }
+};
 
 // ---------------------------------------------------------------------------
 // The fused marching kernel.
@@ -772,12 +1232,7 @@ __global__ void __launch_bounds__(BX) k_march(const Phys<typename C::value_t> P,
     const int sm = slot_of(r - 1), sp = slot_of(r + 1);
     for (int j = tid - 1; j <= w; j += BX) {
       const int c = j + R;
-      const T ph = sphi[s][c];
-      const T lap = (((sphi[s][c + 1] - ph) + (sphi[s][c - 1] - ph)) + ((sphi[sp][c] - ph) + (sphi[sm][c] - ph))) *
-                        T(2.0 / 3.0) +
-                    (((sphi[sp][c + 1] - ph) + (sphi[sm][c - 1] - ph)) + ((sphi[sp][c - 1] - ph) + (sphi[sm][c + 1] - ph))) *
-                        T(1.0 / 6.0);
-      smu[s][j + 1] = P.beta4 * (ph - P.phiA) * (ph - P.phiB) * (ph - P.phibar) - P.kappa * lap;
+      smu[s][j + 1] = chem_pot_rows<C, true>(P, &sphi[sm][c], &sphi[s][c], &sphi[sp][c]);
     }
   };
   // -- CH: mirror ghosts of mu (x walls after make_mu, y walls whole rows)
@@ -884,30 +1339,10 @@ __global__ void __launch_bounds__(BX) k_march(const Phys<typename C::value_t> P,
     if (active) {
       const int sm = slot_of(y - 1), s0 = slot_of(y), sp = slot_of(y + 1);
       const int c = tid + R;
-      T phi9[9];
-      phi9[0] = sphi[s0][c];
-      phi9[1] = sphi[s0][c + 1];
-      phi9[2] = sphi[sp][c];
-      phi9[3] = sphi[s0][c - 1];
-      phi9[4] = sphi[sm][c];
-      phi9[5] = sphi[sp][c + 1];
-      phi9[6] = sphi[sp][c - 1];
-      phi9[7] = sphi[sm][c - 1];
-      phi9[8] = sphi[sm][c + 1];
-      T mu9[9];
-      if (MODEL == MODEL_CH) {
-        const int cm = tid + 1;
-        mu9[0] = smu[s0][cm];
-        mu9[1] = smu[s0][cm + 1];
-        mu9[2] = smu[sp][cm];
-        mu9[3] = smu[s0][cm - 1];
-        mu9[4] = smu[sm][cm];
-        mu9[5] = smu[sp][cm + 1];
-        mu9[6] = smu[sp][cm - 1];
-        mu9[7] = smu[sm][cm - 1];
-        mu9[8] = smu[sm][cm + 1];
-      }
-      node_update<C, MODEL, MODE>(P, B, x, y, phi9, mu9, fq[0], g, h, uin, vin, pin);
+      Stencil<C, MODEL, true> st;  // the moment form in both types
+      st.phi_rows(&sphi[sm][c], &sphi[s0][c], &sphi[sp][c]);
+      if (MODEL == MODEL_CH) st.mu_rows(&smu[sm][tid + 1], &smu[s0][tid + 1], &smu[sp][tid + 1]);
+      st.template update<MODE, false>(P, B, x, y, fq[0], g, h, uin, vin, pin);
     }
     // advance the queue of pulled f
 #pragma unroll
@@ -918,7 +1353,377 @@ __global__ void __launch_bounds__(BX) k_march(const Phys<typename C::value_t> P,
 }
 
 // ---------------------------------------------------------------------------
-// TMA-staged fused step (Allen-Cahn, MODE_STEP): the hot path.
+// One pass over the grid, one node per thread: a block owns a tile of bw x bh
+// nodes, forms phi (Cahn-Hilliard: and mu_phi) of the tile and its halo ring in
+// shared memory straight from pulls of the planes, and updates its nodes.
+//
+// What it replaced, a march of 128- to 160-column strips over staged rows, moved
+// the same bytes but held 16 to 20 warps per SM that waited on each other at
+// every row, needed eight rows per block to pay for its start, and left most
+// SMs idle on small grids.  Here all 23 values of a node are in flight at once,
+// blocks are independent, 24 (FP32) to 32 (Cahn-Hilliard) warps per SM cover the
+// latency, and every SM gets nodes.  The ring is pulled again by the neighbouring
+// blocks, from L2 (DRAM moves 178 bytes per FP32 node update; the algorithmic
+// 184 less what L2 keeps).
+// What bounds it: FP32 by DRAM and its latency (4096^2: 522 us a step, 5.9 TB/s,
+// 0.87 of a copy); FP64 by the FP64 pipe (85 % busy, 209 instructions per node);
+// small grids by one chain of launch, pull, barrier, update and store (4 us).
+// Measured, us a step, before -> now: FP32 128^2 20.4 -> 3.6, 300 x 150 21.8 ->
+// 4.7, 512^2 27.6 -> 9.7, 2048 x 1024 77.8 -> 70.3, 4096^2 558 -> 524, 8192^2
+// 2132 -> 2075, 16384^2 8324 -> 8259; FP64 4 x 256 857 -> 12, 128^2 103 -> 14.5,
+// 2048^2 2842 -> 1646 (with node_update); FP32 Cahn-Hilliard 128^2 23.9 -> 4.7,
+// 4096^2 717 -> 598.
+//
+// Interior tiles address everything from block-uniform bases with one 32-bit
+// offset per node (675 instructions per warp of nodes; 948 with per-node 64-bit
+// addresses and wrap tests, which was issue-bound).  Tiles wider than 32 columns
+// and flatter than 4 rows pull more of the ring than they save (4096^2: 64 x 4
+// 543 us, 128 x 1 617).  Kept to 32 columns, a warp is one row.
+// ---------------------------------------------------------------------------
+// Threads and resident blocks per SM it is compiled for.
+constexpr int TILE_THREADS = 256;
+template <typename T, int MODEL>
+struct TileCfg {
+  static constexpr int blocks = sizeof(T) == 8 ? 2 : (MODEL == MODEL_CH ? 4 : 3);
+};
+
+// Addresses of a tile that lies, with everything it pulls, inside the stored
+// rows (no wall and no periodic wrap in y; in x the row pads hold the wrapped
+// columns): one 32-bit offset per node from block-uniform bases, nine planes'
+// pulls as uniform displacements of it.
+template <typename T>
+struct TileAddr {
+  const unsigned char* base;  // set pointer of tile corner (-PADR rows, -XPAD columns)
+  static constexpr int PADR = 3;
+  int pitch;
+  __device__ __forceinline__ TileAddr(const void* set, const Phys<T>& P, int x0, int y0)
+      : base(static_cast<const unsigned char*>(set) + ((long long)(y0 - PADR) * 9 * P.pitch + x0) * (long long)sizeof(T)),
+        pitch(P.pitch) {}
+  // byte offset of the node (cx, cy) of the tile
+  static __device__ __forceinline__ uint32_t node(int cx, int cy, int pitch) {
+    return (uint32_t)(((cy + PADR) * 9 * pitch + cx + XPAD) * (int)sizeof(T));
+  }
+  template <int I>
+  __device__ __forceinline__ T pulled(uint32_t o) const {
+    constexpr int cx[9] = {0, 1, 0, -1, 0, 1, -1, -1, 1};
+    constexpr int cy[9] = {0, 0, 1, 0, -1, 1, 1, -1, -1};
+    const unsigned char* b = base + ((long long)(I - 9 * cy[I]) * pitch - cx[I]) * (long long)sizeof(T);
+    return *reinterpret_cast<const T*>(b + o);
+  }
+  __device__ __forceinline__ void pull(uint32_t o, T v[9]) const {
+    v[0] = pulled<0>(o), v[1] = pulled<1>(o), v[2] = pulled<2>(o), v[3] = pulled<3>(o), v[4] = pulled<4>(o);
+    v[5] = pulled<5>(o), v[6] = pulled<6>(o), v[7] = pulled<7>(o), v[8] = pulled<8>(o);
+  }
+};
+
+// Outputs of a node of such a tile (plain storage, STEP), from the same kind
+// of offsets: o9 for the population sets, o5 for the history.
+template <typename T>
+struct TileSink {
+  const Phys<T>& P;
+  const Bufs<T>& B;
+  unsigned char *f, *g, *h;  // block-uniform
+  uint32_t o9, o5;
+  int x, y;
+  __device__ __forceinline__ void hist(T a, T b, T c, T d, T e, T phi) const {
+    const long long pc = (long long)P.pitch * (long long)sizeof(T);
+    *reinterpret_cast<T*>(h + o5) = a;
+    *reinterpret_cast<T*>(h + pc + o5) = b;
+    *reinterpret_cast<T*>(h + 2 * pc + o5) = c;
+    *reinterpret_cast<T*>(h + 3 * pc + o5) = d;
+    *reinterpret_cast<T*>(h + 4 * pc + o5) = e;
+    if (B.phi_prev) B.phi_prev[ix(P, 1, 0, x, y)] = phi;
+  }
+  __device__ __forceinline__ T* macro() const { return nullptr; }
+  __device__ __forceinline__ void pops(int set, const T v[9], T, bool) const {
+    unsigned char* const s = set ? g : f;
+    const long long pc = (long long)P.pitch * (long long)sizeof(T);
+#pragma unroll
+    for (int i = 0; i < 9; ++i) *reinterpret_cast<T*>(s + i * pc + o9) = v[i];
+  }
+};
+
+// The update of a tile that reaches a solid obstacle (Allen-Cahn STEP; a solid
+// node within 3 nodes of the tile): phi of the fluid nodes up to two nodes out
+// from mask-aware pulls, then the neutral-wetting value at the solid nodes of
+// the ring around the tile (the mean over their fluid axis neighbours, or, with
+// none, over their fluid diagonal neighbours; zero at solid nodes no fluid node
+// reads), then the wall ghosts, all in shared memory, so that an obstacle costs
+// no pass and no plane of its own.  sp: [bh + 4][bw + 4].
+template <class C, bool UR, typename T = typename C::value_t>
+__device__ __forceinline__ void tile_near_obstacle(const Phys<T>& P, const Bufs<T>& B, T* sp, int x0, int y0, int w,
+                                                   int hgt, int tx, int ty, int tid, int nth) {
+  const int nx = P.nx, ny = P.ny, pw = blockDim.x + 4;
+  const bool wx = P.wall_x != 0, wy = P.wall_y != 0;
+  // the node (cx, cy) of the tile in the grid; false beyond a wall
+  auto node_at = [&](int cx, int cy, int& xx, int& yy) {
+    xx = x0 + cx, yy = y0 + cy;
+    if ((wx && (xx < 0 || xx >= nx)) || (wy && (yy < 0 || yy >= ny))) return false;
+    xx = xx < 0 ? xx + nx : (xx >= nx ? xx - nx : xx);
+    yy = yy < 0 ? yy + ny : (yy >= ny ? yy - ny : yy);
+    return true;
+  };
+  int xx, yy;
+  for (int k = tid; k < (w + 4) * (hgt + 4); k += nth) {
+    const int r = k / (w + 4), c = k - r * (w + 4);
+    if (!node_at(c - 2, r - 2, xx, yy)) continue;
+    const unsigned m = P.obs[(long long)yy * nx + xx];
+    if ((m >> OBS_SOLID) & 1u) continue;
+    T v[9];
+    pull9_obs<C>(B.fin, P, 0, xx, yy, m, v);
+    sp[r * pw + c] = sum9(v);
+  }
+  __syncthreads();
+  for (int k = tid; k < (w + 2) * (hgt + 2); k += nth) {
+    const int r = k / (w + 2), c = k - r * (w + 2);
+    if (!node_at(c - 1, r - 1, xx, yy)) continue;
+    const unsigned m = P.obs[(long long)yy * nx + xx];
+    if (!((m >> OBS_SOLID) & 1u)) continue;
+    constexpr int cx[9] = {0, 1, 0, -1, 0, 1, -1, -1, 1};
+    constexpr int cy[9] = {0, 0, 1, 0, -1, 1, 1, -1, -1};
+    constexpr int op[9] = {0, 3, 4, 1, 2, 7, 8, 5, 6};
+    T* const q = sp + (r + 1) * pw + c + 1;
+    T val = T(0);
+#pragma unroll
+    for (int k0 = 1; k0 <= 5; k0 += 4) {
+      T sum = T(0);
+      int n = 0;
+#pragma unroll
+      for (int j = k0; j < k0 + 4; ++j)
+        if (!((m >> (op[j] - 1)) & 1u)) sum += q[cy[j] * pw + cx[j]], ++n;
+      if (n > 0) {
+        val = sum / T(n);
+        break;
+      }
+    }
+    *q = val;
+  }
+  __syncthreads();
+  if (wx && (x0 == 0 || x0 + w == nx)) {
+    for (int r = tid; r < hgt + 2; r += nth) {
+      T* const q = sp + (r + 1) * pw + 2;
+      if (x0 == 0) q[-1] = wall_ghost(P, SIDE_LEFT, q[0], q[1]);
+      if (x0 + w == nx) q[w] = wall_ghost(P, SIDE_RIGHT, q[w - 1], q[w - 2]);
+    }
+    __syncthreads();
+  }
+  if (wy && (y0 == 0 || y0 + hgt == ny)) {
+    for (int c = tid; c < w + 2; c += nth) {
+      T* const q = sp + 2 * pw + c + 1;
+      if (y0 == 0) q[-pw] = wall_ghost(P, SIDE_BOTTOM, q[0], q[pw]);
+      if (y0 + hgt == ny) q[hgt * pw] = wall_ghost(P, SIDE_TOP, q[(hgt - 1) * pw], q[(hgt - 2) * pw]);
+    }
+    __syncthreads();
+  }
+  if (tx >= w || ty >= hgt) return;
+  const int x = x0 + tx, y = y0 + ty;
+  const unsigned m = P.obs[(long long)y * nx + x];
+  const NodeSink<C, MODE_STEP> out{P, B, x, y};
+  T f[9], g[9], h[5];
+  pull9_obs<C>(B.fin, P, 0, x, y, m, f);  // zeros at a solid node
+  if ((m >> OBS_SOLID) & 1u) {
+    out.hist(T(0), T(0), T(0), T(0), T(0), T(0));
+    out.pops(0, f, T(0), true);
+    out.pops(1, f, T(0), false);
+    return;
+  }
+  pull9_obs<C>(B.gin, P, 1, x, y, m, g);
+#pragma unroll
+  for (int k = 0; k < 5; ++k) h[k] = B.hist[ix(P, 5, k, x, y)];
+  Stencil<C, MODEL_AC> st;
+  const T* const q = sp + (ty + 2) * pw + tx + 2;
+  st.phi_rows(q - pw, q, q + pw);
+  st.template update<MODE_STEP, UR>(P, out, f, g, h, T(0), T(0), T(0));
+}
+
+// OBS: solid obstacles (Allen-Cahn STEP); tiles flagged in P.obs_near take the
+// path above, the others the plain one.  MOM: the node update's moment form.
+template <class C, int MODEL, int MODE, bool UR, bool OBS = false, bool MOM = sizeof(typename C::value_t) == 4>
+__global__ void __launch_bounds__(TILE_THREADS, (TileCfg<typename C::value_t, MODEL>::blocks))
+    k_tile(const Phys<typename C::value_t> P, const Bufs<typename C::value_t> B) {
+  using T = typename C::value_t;
+  constexpr int R = (MODEL == MODEL_CH) ? 2 : 1;  // phi halo radius
+  extern __shared__ __align__(16) unsigned char tile_smem[];
+  const int bw = blockDim.x, bh = blockDim.y;
+  const int pw = bw + 2 * R, mw = bw + 2;
+  T* const sp = reinterpret_cast<T*>(tile_smem);  // [bh + 2R][pw]
+  T* const sm = sp + pw * (bh + 2 * R);           // CH: [bh + 2][mw]
+  const int tx = threadIdx.x, ty = threadIdx.y;
+  const int tid = ty * bw + tx, nth = bw * bh;
+  const int nx = P.nx, ny = P.ny;
+  const int x0 = blockIdx.x * bw, y0 = blockIdx.y * bh;
+  const int w = min(bw, nx - x0), hgt = min(bh, ny - y0);
+  const bool active = tx < w && ty < hgt;
+  const int x = x0 + tx, y = y0 + ty;
+  const bool wx = P.wall_x != 0, wy = P.wall_y != 0;
+  // everything the tile pulls lies in the stored rows, without a ghost
+  const bool inner = MODE != MODE_INIT && w == bw && hgt == bh && y0 > R && y0 + bh + R < ny &&
+                     (!wx || (x0 > R && x0 + bw + R < nx));
+
+  // a programmatic dependent of the kernel before it, like the marching steps
+  asm volatile("griddepcontrol.launch_dependents;");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+
+  if constexpr (OBS) {
+    if (P.obs_near[blockIdx.y * gridDim.x + blockIdx.x]) {
+      tile_near_obstacle<C, UR>(P, B, sp, x0, y0, w, hgt, tx, ty, tid, nth);
+      return;
+    }
+  }
+  T f[9] = {T(0), T(0), T(0), T(0), T(0), T(0), T(0), T(0), T(0)};
+  T g[9] = {T(0), T(0), T(0), T(0), T(0), T(0), T(0), T(0), T(0)};
+  T h[5] = {T(0), T(0), T(0), T(0), T(0)};
+  T uin = T(0), vin = T(0), pin = T(0);
+  const uint32_t o9 = TileAddr<T>::node(tx, ty, P.pitch);
+  const uint32_t o5 = (uint32_t)((ty * 5 * P.pitch + tx) * (int)sizeof(T));
+  unsigned char* const hb = reinterpret_cast<unsigned char*>(B.hist + ix(P, 5, 0, x0, y0));
+  if (inner) {
+    const TileAddr<T> F(B.fin, P, x0, y0), G(B.gin, P, x0, y0);
+    // the halo ring, a warp's share at a time: R rows below and R above (columns
+    // [0, bw), bw <= 32), then R columns on either side of all bh + 2R rows
+    const int shares = 2 * R + (2 * R * (bh + 2 * R) + 31) / 32, warps = (nth + 31) >> 5;
+    auto place = [&](int k, int& cx, int& cy) {
+      cx = tid & 31;
+      if (k < 2 * R) {
+        cy = k < R ? k - R : bh + k - R;
+        return cx < bw;
+      }
+      const int q = (k - 2 * R) * 32 + cx;
+      cy = q / (2 * R) - R;
+      cx = q % (2 * R);
+      cx = cx < R ? cx - R : bw + cx - R;
+      return cy < bh + R;
+    };
+    auto load_gh = [&]() {
+      G.pull(o9, g);
+      if (MODE == MODE_STEP || MODE == MODE_MACRO) {
+        const long long pc = (long long)P.pitch * (long long)sizeof(T);
+#pragma unroll
+        for (int i = 0; i < 5; ++i) h[i] = *reinterpret_cast<const T*>(hb + i * pc + o5);
+      }
+    };
+    T v[9];
+    int k = tid >> 5, cx, cy;
+    if constexpr (MODEL == MODEL_AC) {
+      // the first share's loads go out before the thread's own nodes', whose
+      // latency they share (4096^2 FP32: 522 us a step; after f's: 610)
+      const bool on = k < shares && place(k, cx, cy);
+      if (on) F.pull(TileAddr<T>::node(cx, cy, P.pitch), v);
+      F.pull(o9, f);
+      load_gh();
+      if (on) sp[(cy + R) * pw + cx + R] = sum9(v);
+      k += warps;
+    } else {
+      // a ring two nodes wide wants the registers: its loads before g's
+      F.pull(o9, f);
+    }
+    for (; k < shares; k += warps) {
+      if (!place(k, cx, cy)) continue;
+      F.pull(TileAddr<T>::node(cx, cy, P.pitch), v);
+      sp[(cy + R) * pw + cx + R] = sum9(v);
+    }
+    if constexpr (MODEL == MODEL_CH) load_gh();
+    sp[(ty + R) * pw + tx + R] = sum9(f);
+    __syncthreads();
+  } else {
+    if (active) {
+      if (MODE == MODE_INIT) {
+        const long long di = (long long)y * nx + x;
+        if (B.iux) uin = T(B.iux[di]);
+        if (B.iuy) vin = T(B.iuy[di]);
+        if (B.ip) pin = T(B.ip[di]);
+      } else {
+        pull9<C>(B.fin, P, 0, x, y, f);
+        pull9<C>(B.gin, P, 1, x, y, g);
+        if (MODE == MODE_STEP || MODE == MODE_MACRO) {
+#pragma unroll
+          for (int k = 0; k < 5; ++k) h[k] = B.hist[ix(P, 5, k, x, y)];
+        }
+      }
+    }
+    // the halo ring (in the domain, or wrapped): R rows below and above over the
+    // widened columns, then R columns on either side
+    const int row_cells = R * (w + 2 * R), ring = 2 * row_cells + 2 * R * hgt;
+    for (int k = tid; k < ring; k += nth) {
+      int cx, cy;
+      if (k < 2 * row_cells) {
+        const int r = k / (w + 2 * R);
+        cx = k - r * (w + 2 * R) - R;
+        cy = r < R ? r - R : hgt + (r - R);
+      } else {
+        const int q = k - 2 * row_cells, r = q / (2 * R), c = q - r * 2 * R;
+        cy = r;
+        cx = c < R ? c - R : w + (c - R);
+      }
+      int xx = x0 + cx, yy = y0 + cy;
+      if ((wx && (xx < 0 || xx >= nx)) || (wy && (yy < 0 || yy >= ny))) continue;  // ghosts follow
+      xx = xx < 0 ? xx + nx : (xx >= nx ? xx - nx : xx);
+      yy = yy < 0 ? yy + ny : (yy >= ny ? yy - ny : yy);
+      sp[(cy + R) * pw + cx + R] = phi_at<C, MODE>(P, B, xx, yy);
+    }
+    if (active) sp[(ty + R) * pw + tx + R] = MODE == MODE_INIT ? T(B.iphi[(long long)y * nx + x]) : sum9(f);
+    __syncthreads();
+    // wetting ghosts: the column beyond an x wall on every row the tile and its
+    // halo hold, then the row beyond a y wall over the widened columns.  cl, cr,
+    // rb, rt: their places relative to the tile (block-uniform; a Cahn-Hilliard
+    // tile that ends one node short of a wall holds the ghosts too, for mu_phi
+    // of the node between)
+    const int cl = -1 - x0, cr = nx - x0, rb = -1 - y0, rt = ny - y0;
+    const bool has_l = wx && cl >= -R, has_r = wx && cr < w + R;
+    const bool has_b = wy && rb >= -R, has_t = wy && rt < hgt + R;
+    if (has_l || has_r) {
+      for (int r = tid; r < hgt + 2 * R; r += nth) {
+        T* const q = sp + r * pw + R;
+        if (has_l) q[cl] = wall_ghost(P, SIDE_LEFT, q[cl + 1], q[cl + 2]);
+        if (has_r) q[cr] = wall_ghost(P, SIDE_RIGHT, q[cr - 1], q[cr - 2]);
+      }
+      __syncthreads();
+    }
+    if (has_b || has_t) {
+      for (int c = tid; c < w + 2 * R; c += nth) {
+        T* const q = sp + R * pw + c;
+        if (has_b) q[rb * pw] = wall_ghost(P, SIDE_BOTTOM, q[(rb + 1) * pw], q[(rb + 2) * pw]);
+        if (has_t) q[rt * pw] = wall_ghost(P, SIDE_TOP, q[(rt - 1) * pw], q[(rt - 2) * pw]);
+      }
+      __syncthreads();
+    }
+  }
+  if (MODEL == MODEL_CH) {
+    // mu_phi on the tile and one node around it; beyond walls the mirror value
+    const bool gl = wx && x0 == 0, gr = wx && x0 + w == nx, gb = wy && y0 == 0, gt = wy && y0 + hgt == ny;
+    for (int k = tid; k < mw * (hgt + 2); k += nth) {
+      const int r = k / mw, c = k - r * mw;  // node (x0 + c - 1, y0 + r - 1)
+      if (c >= w + 2) continue;
+      const int cc = (gl && c == 0) ? 1 : ((gr && c == w + 1) ? w : c);
+      const int rr = (gb && r == 0) ? 1 : ((gt && r == hgt + 1) ? hgt : r);
+      const T* const q = sp + (rr + R - 1) * pw + cc + R - 1;
+      sm[r * mw + c] = chem_pot_rows<C>(P, q - pw, q, q + pw);
+    }
+    __syncthreads();
+  }
+  if (!active) return;
+  Stencil<C, MODEL, MOM> st;
+  const T* const q = sp + (ty + R) * pw + tx + R;
+  st.phi_rows(q - pw, q, q + pw);
+  if (MODEL == MODEL_CH) {
+    const T* const m = sm + (ty + 1) * mw + tx + 1;
+    st.mu_rows(m - mw, m, m + mw);
+  }
+  if constexpr (MODE == MODE_STEP) {
+    // no periodic copies to write: the tile does not touch the pads' columns
+    if (inner && (wx || (x0 >= XPAD && x0 + bw <= nx - XPAD))) {
+      const long long org = ((long long)(y0 - TileAddr<T>::PADR) * 9 * P.pitch + x0) * (long long)sizeof(T);
+      const TileSink<T> out{P, B, static_cast<unsigned char*>(B.fout) + org, static_cast<unsigned char*>(B.gout) + org,
+                            hb, o9, o5, x, y};
+      st.template update<MODE, UR>(P, out, f, g, h, uin, vin, pin);
+      return;
+    }
+  }
+  st.template update<MODE, UR>(P, B, x, y, f, g, h, uin, vin, pin);
+}
+
+// ---------------------------------------------------------------------------
+// TMA-staged fused step (Allen-Cahn, MODE_STEP): the 16-bit deviation codecs.
 //
 // Same per-node arithmetic as k_march, with the population rows brought in
 // by the Tensor Memory Accelerator: one elected thread issues, per source
@@ -940,9 +1745,7 @@ struct Seg {
 };
 // Rings: f rows y-1 .. y+2 are live while row y is processed (pulls of row y,
 // phi of row y+1) and DF more rows are in flight; g rows y-1 .. y+1 are live
-// and DG more are in flight.  SLIM: the pulled f of row y is kept in
-// registers from phi's pass over that row, so f row y-1 is not needed and
-// the f ring is one row shorter.
+// and DG more are in flight.
 // phi ring of the TMA step: rows y-2 .. y+1 can be in use at once (slower
 // threads of the previous march step read y-2 .. y while row y+1 is formed)
 constexpr int TRING = 4;
@@ -950,11 +1753,11 @@ __host__ __device__ constexpr int tslot(int r) { return (r + 2 * TRING) & (TRING
 
 // A staged row slot holds the segment of each of the nine planes: plane 0
 // (SEG elements of B0 bytes) then planes 1..8 (SEG elements of BI bytes).
-template <class C, int TBX, int DF, int DG, bool SLIM = false>
+template <class C, int TBX, int DF, int DG>
 struct TmaLayout {
   using T = typename C::value_t;
   static constexpr int SEG = Seg<TBX>::value;
-  static constexpr int RF = (SLIM ? 3 : 4) + DF, RG = 3 + DG;
+  static constexpr int RF = 4 + DF, RG = 3 + DG;
   static constexpr size_t P0 = (size_t)SEG * C::B0;   // bytes of plane 0's segment
   static constexpr size_t PI = (size_t)SEG * C::BI;   // bytes of each other plane's segment
   static constexpr size_t SLOT = P0 + 8 * PI;
@@ -1083,41 +1886,25 @@ __device__ __forceinline__ void pull_staged_obs(const unsigned char* rm, const u
   out[8] = (m & 128u) ? stg_ld<C, SEG>(r0, 6, c, r2, is) : stg_ld<C, SEG>(rp, 8, c - 1, r2, is);
 }
 
-// Launch shape of the TMA step per storage codec: strip width, rows staged
-// ahead of need (f, g), resident threads per SM it is compiled for
-// (registers), and whether the f pulled for phi of row y+1 is kept in
-// registers for that row's collision instead of being pulled again.
-//   FP32: 160 columns, f one row ahead, g two, 4 blocks (20 warps) per SM:
-//         shared memory (56 KB a block) is the occupancy limit.  f is kept
-//         from phi's pass (SLIM), and the f slot that frees holds the extra g
-//         row.
-//   FP64: 160 columns, one row ahead, one block per SM (registers).
-//   16-bit deviations: 128 columns, two rows ahead, 6 blocks (24 warps) per
-//         SM; the rows are 44 % smaller, so more blocks fit, and keeping f
-//         saves the second decode.
-// Measured on the 16384^2 step (GLUPS): FP32 160/1/1 29.5-30.6 against 128
-// to 256 columns, deeper staging or more blocks 24.9-28.2.  FP16 deviations
-// 128/2/2 x6 with kept f 34.4; 160/1/1 x4 30.3; 160/2/2 x5 32.3, with kept
-// f 33.4; 96/2/2 x8 33.1; 256/2/2 x3 32.5; history staged by TMA or copies
-// issued from every warp 27-29.  Keeping f in FP32 too, which frees the f
-// ring's row y-1 and lets f be staged two rows ahead in the same shared
-// memory (the segment's first phi row then pulled from global memory):
-// FP32 30.6 (unchanged), FP16 deviations 32.3 (register spills); the same
-// ring with g staged two rows ahead instead: FP32 32.0.  Without the per-row
-// block barrier (each warp keeping its own phi ring and re-forming its halo
-// columns, row slots recycled through per-slot mbarriers that every warp
-// arrives on): FP32 29.2, FP16 deviations 27.2, so the barrier stays.
-// FP16 deviations with the f ring starting at row y0-1 as in FP32 and 7
-// blocks (28 warps) per SM: 33.9 against 34.8 (46 B of spills at 72
-// registers).
+// Launch shape of the TMA step: strip width, rows staged ahead of need (f, g),
+// resident threads per SM it is compiled for (registers).  128 columns, two
+// rows ahead, 6 blocks (24 warps) per SM; the f pulled for phi of row y+1 is
+// kept in registers for that row's collision (a second decode saved).
+// Measured on the 16384^2 step, FP16 deviations (GLUPS): 34.4; 160/1/1 x4
+// 30.3; 160/2/2 x5 32.3, with kept f 33.4; 96/2/2 x8 33.1; 256/2/2 x3 32.5;
+// history staged by TMA or copies issued from every warp 27-29; without the
+// per-row block barrier (each warp keeping its own phi ring and re-forming
+// its halo columns, row slots recycled through per-slot mbarriers that every
+// warp arrives on) 27.2; the f ring starting at row y0-1 and 7 blocks per SM
+// 33.9 against 34.8 (spills at 72 registers).  One node per thread, as k_tile:
+// 1050 us a step against 531 at 4096^2 (its unaligned 16-bit loads cost as many
+// instructions as FP32 ones and the decode comes on top), though 17 against 35
+// at 512^2; it rounds otherwise, and a grid and its slabs must not take
+// different kernels.
 template <class C>
 struct TmaCfg {
-  static constexpr int TBX = C::dev ? 128 : 160;
-  static constexpr bool fp32 = !C::dev && sizeof(typename C::value_t) == 4;
-  static constexpr int DF = C::dev ? 2 : 1, DG = (C::dev || fp32) ? 2 : 1;
-  static constexpr int threads = C::dev ? 768 : (sizeof(typename C::value_t) == 4 ? 640 : 256);
-  static constexpr bool keep_f = C::dev || fp32;
-  static constexpr bool slim = fp32;
+  static_assert(C::dev, "the plain codecs step with k_tile");
+  static constexpr int TBX = 128, DF = 2, DG = 2, threads = 768;
 };
 
 // VSEG: segments of P.seg_rows rows (small grids) instead of the constant LY.
@@ -1131,9 +1918,7 @@ __global__ void __launch_bounds__(TmaCfg<C>::TBX, TmaCfg<C>::threads / TmaCfg<C>
     k_step_tma(const Phys<typename C::value_t> P, const Bufs<typename C::value_t> B, int* __restrict__ err) {
   using T = typename C::value_t;
   constexpr int TBX = TmaCfg<C>::TBX, DF = TmaCfg<C>::DF, DG = TmaCfg<C>::DG;
-  constexpr bool FK = TmaCfg<C>::keep_f;
-  constexpr bool SLIM = TmaCfg<C>::slim;  // (implies FK) the f ring starts at row y0 - 1
-  using L = TmaLayout<C, TBX, DF, DG, SLIM>;
+  using L = TmaLayout<C, TBX, DF, DG>;
   constexpr int SEG = L::SEG, RF = L::RF, RG = L::RG;
   constexpr int FS = (int)L::SLOT;  // bytes per row slot
   extern __shared__ __align__(128) unsigned char smem[];
@@ -1152,7 +1937,7 @@ __global__ void __launch_bounds__(TmaCfg<C>::TBX, TmaCfg<C>::threads / TmaCfg<C>
   const bool active = tid < w;
   const int x = x0 + tid;
   const bool wx = P.wall_x != 0, wy = P.wall_y != 0;
-  const int fbase = y0 - (SLIM ? 1 : 2), gbase = y0 - 1;  // first staged f / g row
+  const int fbase = y0 - 2, gbase = y0 - 1;  // first staged f / g row
   // bytes copied per plane segment: [x0 - XPAD, x0 + w + XPAD) rounded up to 16
   const uint32_t seg0 = (uint32_t)((((w + 2 * XPAD) * C::B0 + 15) / 16) * 16);
   const uint32_t segI = (uint32_t)((((w + 2 * XPAD) * C::BI + 15) / 16) * 16);
@@ -1195,19 +1980,6 @@ __global__ void __launch_bounds__(TmaCfg<C>::TBX, TmaCfg<C>::threads / TmaCfg<C>
       bulk_g2s(slot + L::P0 + (i - 1) * L::PI, row + pop_plane_off<C>(P.pitch, i) + (long long)x0 * C::BI,
                segI, bar);
   };
-  // the same issued by lanes 0..8 of warp 0, one plane each (every lane of
-  // warp 0 calls it; tid is the lane there)
-  auto stage_lanes = [&](const void* src, unsigned char* slot, uint64_t* bar, int r) {
-    if ((r < 0 || r >= ny) && wy) {
-      if (tid == 0) mbar_arrive(bar);
-      return;
-    }
-    const unsigned char* row = static_cast<const unsigned char*>(src) + (long long)wrap_row(r) * RB;
-    if (tid == 0) mbar_arrive_expect_tx(bar, seg0 + 8u * segI);
-    if (tid < 9)
-      bulk_g2s(slot + (tid ? L::P0 + (tid - 1) * L::PI : 0),
-               row + pop_plane_off<C>(P.pitch, tid) + (long long)x0 * (tid ? C::BI : C::B0), tid ? segI : seg0, bar);
-  };
   auto fslot = [&](int r) { return sf + ((r - fbase) % RF) * FS; };
   auto gslot = [&](int r) { return sg + ((r - gbase) % RG) * FS; };
   auto wait_f = [&](int r) {
@@ -1222,11 +1994,11 @@ __global__ void __launch_bounds__(TmaCfg<C>::TBX, TmaCfg<C>::threads / TmaCfg<C>
   // phi of row r (in the domain, or wrapped) into the phi ring: own column,
   // left halo (thread 0), right halo (thread w - 1); x-wall ghosts from the
   // thread's own phi and a second pull of the neighbouring column.
-  T fnext[9];  // FK: the pulled f of the last phi row made with keep set
-  unsigned mnext = 0;  // OBS and FK: the link word of that row's node
+  T fnext[9];  // the pulled f of the last phi row made with keep set
+  unsigned mnext = 0;  // OBS: the link word of that row's node
   // OBS: phi of row r from the filled plane (x-wall ghosts as in the plain
   // step, from the plane's columns 0, 1 and nx-1, nx-2).  The plane values
-  // and the link word (FK) of a row are loaded one march step before the
+  // and the link word of a row are loaded one march step before the
   // row is formed, so that their latency overlaps a node update.
   int pre_r = INT_MIN;  // the row whose values the pre_ registers hold
   T pre_c = T(0), pre_l0 = T(0), pre_l1 = T(0), pre_r0 = T(0), pre_r1 = T(0);
@@ -1238,7 +2010,7 @@ __global__ void __launch_bounds__(TmaCfg<C>::TBX, TmaCfg<C>::threads / TmaCfg<C>
     const int rr = wrap_row(r);
     const T* pr = B.phis + ix(P, 1, 0, 0, rr);
     pre_c = pr[x];
-    if (FK) pre_m = P.obs[(long long)rr * nx + x];
+    pre_m = P.obs[(long long)rr * nx + x];
     if (tid == 0) {
       pre_l0 = x0 > 0 ? pr[x0 - 1] : (!wx ? pr[nx - 1] : pr[0]);
       if (wl) pre_l1 = pr[1];
@@ -1248,7 +2020,7 @@ __global__ void __launch_bounds__(TmaCfg<C>::TBX, TmaCfg<C>::threads / TmaCfg<C>
       if (wr) pre_r1 = pr[nx - 2];
     }
   };
-  // returns the link word of row r's node (FK)
+  // returns the link word of row r's node
   auto phi_row_plane = [&](int r) -> unsigned {
     if (pre_r != r) plane_load(r);
     T* dst = sp + tslot(r) * (TBX + 2);
@@ -1268,7 +2040,7 @@ __global__ void __launch_bounds__(TmaCfg<C>::TBX, TmaCfg<C>::threads / TmaCfg<C>
     T* dst = sp + tslot(r) * (TBX + 2);
     if (OBS && near) {
       const unsigned m = phi_row_plane(r);
-      if (FK && keep && active) {
+      if (keep && active) {
         mnext = m;
         pull_staged_obs<C, SEG>(rm, r0, rp, tid + XPAD, mnext, rf2, isf, fnext);
       }
@@ -1282,7 +2054,7 @@ __global__ void __launch_bounds__(TmaCfg<C>::TBX, TmaCfg<C>::threads / TmaCfg<C>
       pull_staged<C, SEG>(rm, r0, rp, tid + XPAD, false, false, false, false, rf2, isf, v);
     const T ph = sum9(v);
     dst[tid + 1] = ph;
-    if (FK && keep) {
+    if (keep) {
 #pragma unroll
       for (int i = 0; i < 9; ++i) fnext[i] = v[i];
     }
@@ -1310,33 +2082,6 @@ __global__ void __launch_bounds__(TmaCfg<C>::TBX, TmaCfg<C>::threads / TmaCfg<C>
     }
   };
   auto phi_row = [&](int r) { phi_row_at(r, fslot(r - 1), fslot(r), fslot(r + 1), r == y0); };
-  // SLIM: phi of row y0 - 1 (in the domain or wrapped) from pulls of the
-  // global planes, since its f rows are not staged.
-  auto phi_row_global = [&](int r) {
-    if (OBS && near) {
-      phi_row_plane(r);
-      return;
-    }
-    const int rr = wrap_row(r);
-    T* dst = sp + tslot(r) * (TBX + 2);
-    if (!active) return;
-    const T ph = phi_at<C, MODE_STEP>(P, B, x, rr);
-    dst[tid + 1] = ph;
-    if (tid == 0) {
-      T hv;
-      if (x0 > 0) hv = phi_at<C, MODE_STEP>(P, B, x0 - 1, rr);
-      else if (!wx) hv = phi_at<C, MODE_STEP>(P, B, nx - 1, rr);
-      else hv = wall_ghost(P, SIDE_LEFT, ph, phi_at<C, MODE_STEP>(P, B, 1, rr));
-      dst[0] = hv;
-    }
-    if (tid == w - 1) {
-      T hv;
-      if (x0 + w < nx) hv = phi_at<C, MODE_STEP>(P, B, x0 + w, rr);
-      else if (!wx) hv = phi_at<C, MODE_STEP>(P, B, 0, rr);
-      else hv = wall_ghost(P, SIDE_RIGHT, ph, phi_at<C, MODE_STEP>(P, B, nx - 2, rr));
-      dst[w + 1] = hv;
-    }
-  };
   auto ghost_row = [&](int rg, int r1, int r2, int side) {
     T* d = sp + tslot(rg) * (TBX + 2);
     const T* a = sp + tslot(r1) * (TBX + 2);
@@ -1360,10 +2105,7 @@ __global__ void __launch_bounds__(TmaCfg<C>::TBX, TmaCfg<C>::threads / TmaCfg<C>
   for (int r = fbase; r <= min(y0 + (bottom ? 2 : 1), f_last); ++r) ok = wait_f(r) && ok;
   for (int r = gbase; r <= min(y0, g_last); ++r) ok = wait_g(r) && ok;
   for (int r = y0 - 1; r <= y0 + (bottom ? 1 : 0); ++r) {
-    if ((r >= 0 && r < ny) || !wy) {
-      if (SLIM && r == y0 - 1) phi_row_global(r);
-      else phi_row(r);
-    }
+    if ((r >= 0 && r < ny) || !wy) phi_row(r);
   }
   bool failed = __syncthreads_or(!ok);
   if (!failed && bottom) {
@@ -1383,7 +2125,7 @@ __global__ void __launch_bounds__(TmaCfg<C>::TBX, TmaCfg<C>::threads / TmaCfg<C>
   // g row y+1), kept as counters instead of modulo arithmetic.
   auto next = [](int s, int R) { return s + 1 == R ? 0 : s + 1; };
   auto add = [](int s, int k, int R) { return s + k >= R ? s + k - R : s + k; };
-  constexpr int LF0 = SLIM ? 1 : 2;                        // local index of f row y0
+  constexpr int LF0 = 2;                                  // local index of f row y0
   int fR0 = LF0 % RF, gA = 0;                              // f row y0, g row y0-1
   int fW = (LF0 + 2) % RF, fWp = ((LF0 + 2) / RF) & 1;     // f row y0+2
   int gW = 2 % RG, gWp = (2 / RG) & 1;       // g row y0+1 (local 2)
@@ -1392,14 +2134,10 @@ __global__ void __launch_bounds__(TmaCfg<C>::TBX, TmaCfg<C>::threads / TmaCfg<C>
     ok = true;
     if (y + 2 <= f_last) ok = mbar_wait_bounded(&barF[fW], fWp) && ok;
     if (y + 1 <= g_last) ok = mbar_wait_bounded(&barG[gW], gWp) && ok;
-    T f[9];  // pulled f of row y (FK: made with phi of row y)
-    unsigned mc = 0;  // OBS: link word of the node of row y
-    if (FK) {
+    T f[9];  // pulled f of row y (made with phi of row y)
 #pragma unroll
-      for (int i = 0; i < 9; ++i) f[i] = fnext[i];
-      mc = mnext;
-    }
-    const unsigned char* f_m = sf + add(fR0, RF - 1, RF) * FS;  // f row y-1 (not SLIM)
+    for (int i = 0; i < 9; ++i) f[i] = fnext[i];
+    const unsigned mc = mnext;                                  // OBS: link word of the node of row y
     const unsigned char* f_0 = sf + fR0 * FS;                   // f row y
     const unsigned char* f_p = sf + add(fR0, 1, RF) * FS;       // f row y+1
     // phi of row y+1 (a ghost row above a top wall)
@@ -1408,20 +2146,16 @@ __global__ void __launch_bounds__(TmaCfg<C>::TBX, TmaCfg<C>::threads / TmaCfg<C>
     else if (r1 == ny) ghost_row(ny, ny - 1, ny - 2, SIDE_TOP);  // rows ny-1, ny-2 ready since the last barrier
     failed = __syncthreads_or(!ok);
     if (failed) break;
-    // the next rows' copies: from lanes 0..8 of warp 0 for FP32 / FP64 sets
-    // (+0.7 % for the FP32 step), from thread 0 for the 16-bit codec (the
-    // lanes' issue measured 5 % slower there)
-    if (C::dev ? tid == 0 : tid < 32) {
+    // the next rows' copies (from nine lanes, one plane each: 5 % slower)
+    if (tid == 0) {
       fence_proxy_async_smem();
       if (y + 2 + DF <= f_last) {
         const int sl = add(fR0, 2 + DF, RF);
-        if (C::dev) stage(B.fin, sf + sl * FS, &barF[sl], y + 2 + DF);
-        else stage_lanes(B.fin, sf + sl * FS, &barF[sl], y + 2 + DF);
+        stage(B.fin, sf + sl * FS, &barF[sl], y + 2 + DF);
       }
       if (y + 1 + DG <= g_last) {
         const int sl = add(gA, 2 + DG, RG);
-        if (C::dev) stage(B.gin, sg + sl * FS, &barG[sl], y + 1 + DG);
-        else stage_lanes(B.gin, sg + sl * FS, &barG[sl], y + 1 + DG);
+        stage(B.gin, sg + sl * FS, &barG[sl], y + 1 + DG);
       }
     }
     T hn[5] = {T(0), T(0), T(0), T(0), T(0)};
@@ -1451,15 +2185,11 @@ __global__ void __launch_bounds__(TmaCfg<C>::TBX, TmaCfg<C>::threads / TmaCfg<C>
       const bool bym = wy && y == 0, byp = wy && y == ny - 1;
       T g[9];
       if (OBS && near) {
-        if (!FK) mc = P.obs[(long long)y * nx + x];
-        if (!FK) pull_staged_obs<C, SEG>(f_m, f_0, f_p, tid + XPAD, mc, rf2, isf, f);
         pull_staged_obs<C, SEG>(g_m, g_0, g_p, tid + XPAD, mc, rg2, isg, g);
       } else if (edge_x || bym || byp) {  // bounce-back links possible (block-uniform test)
         const bool bxm = wx && x == 0, bxp = wx && x == nx - 1;
-        if (!FK) pull_staged<C, SEG>(f_m, f_0, f_p, tid + XPAD, bxm, bxp, bym, byp, rf2, isf, f);
         pull_staged<C, SEG>(g_m, g_0, g_p, tid + XPAD, bxm, bxp, bym, byp, rg2, isg, g);
       } else {
-        if (!FK) pull_staged<C, SEG>(f_m, f_0, f_p, tid + XPAD, false, false, false, false, rf2, isf, f);
         pull_staged<C, SEG>(g_m, g_0, g_p, tid + XPAD, false, false, false, false, rg2, isg, g);
       }
       if (OBS && near && ((mc >> OBS_SOLID) & 1u)) {  // a solid node: no populations, no history
@@ -1472,7 +2202,7 @@ __global__ void __launch_bounds__(TmaCfg<C>::TBX, TmaCfg<C>::threads / TmaCfg<C>
         for (int k = 0; k < 5; ++k) hb[k * P.pitch] = T(0);
         if (B.phi_prev) B.phi_prev[ix(P, 1, 0, x, y)] = T(0);
       } else {
-        node_update<C, MODEL_AC, MODE_STEP, UR>(P, B, x, y, phi9, phi9, f, g, h, T(0), T(0), T(0));
+        node_update_moments<C, MODEL_AC, MODE_STEP, UR>(P, NodeSink<C, MODE_STEP>{P, B, x, y}, phi9, phi9, f, g, h, T(0), T(0), T(0));
       }
     }
 #pragma unroll
@@ -1768,10 +2498,7 @@ __global__ void __launch_bounds__(TmaChCfg<C>::TBX, TmaChCfg<C>::threads / TmaCh
   };
   // mu_phi (Eq. (5)) at ring column j of a row, from phi rows r-1, r, r+1
   auto mu_at = [&](const T* pm, const T* p0, const T* pp, int j) {
-    const T ph = p0[j];
-    const T lap = (((p0[j + 1] - ph) + (p0[j - 1] - ph)) + ((pp[j] - ph) + (pm[j] - ph))) * T(2.0 / 3.0) +
-                  (((pp[j + 1] - ph) + (pm[j - 1] - ph)) + ((pp[j - 1] - ph) + (pm[j + 1] - ph))) * T(1.0 / 6.0);
-    return P.beta4 * (ph - P.phiA) * (ph - P.phiB) * (ph - P.phibar) - P.kappa * lap;
+    return chem_pot_rows<C>(P, pm + j, p0 + j, pp + j);
   };
   // mu_phi of row r for this warp: its own columns, and the column beyond
   // either end (lane 0 and the last active lane form those again); at an x
@@ -1930,7 +2657,7 @@ __global__ void __launch_bounds__(TmaChCfg<C>::TBX, TmaChCfg<C>::threads / TmaCh
         for (int k = 0; k < 5; ++k) hb[k * P.pitch] = T(0);
         if (B.phi_prev) B.phi_prev[ix(P, 1, 0, x, y)] = T(0);
       } else {
-        node_update<C, MODEL_CH, MODE_STEP, UR>(P, B, x, y, phi9, mu9, f, g, h, T(0), T(0), T(0));
+        node_update_nine<C, MODEL_CH, MODE_STEP, UR>(P, NodeSink<C, MODE_STEP>{P, B, x, y}, phi9, mu9, f, g, h, T(0), T(0), T(0));
       }
     }
 #pragma unroll

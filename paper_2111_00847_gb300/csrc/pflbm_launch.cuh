@@ -1,7 +1,7 @@
 // Definitions of the launch wrappers declared in pflbm_launch.h.
 #pragma once
 
-#include <cmath>
+#include <algorithm>
 
 #include "pflbm_launch.h"
 
@@ -51,38 +51,13 @@ static inline int segment_rows(int nx, int ny, int tbx, int per_sm, int waves = 
   return seg;
 }
 
-// Rows per segment of the FP32 Allen-Cahn step on grids that hold fewer than
-// eight waves of LY-row blocks: the length in [8, LY] with the least
-// modelled time.  A block takes time in proportion to its rows plus two (the
-// rows it re-stages first); blocks run in waves of (SMs x resident blocks),
-// and a partial last wave of this latency-bound kernel costs about half a
-// full wave beyond its share of the blocks.  Measured: 2048 x 1024 picks 23
-// rows (26.2 GLUPS, 23.9 at 8), 4096 x 2048 picks 45 (28.1, 27.4 at 32).
-static inline int segment_rows_waves(int nx, int ny, int tbx, int per_sm) {
-  const long long slots = (long long)device_sm_count() * per_sm;
-  const long long strips = (nx + tbx - 1) / tbx;
-  if (strips * ((ny + LY - 1) / LY) >= 8 * slots) return LY;
-  int pick = LY;
-  double best = 0.0;
-  for (int seg = LY; seg >= 8; --seg) {
-    const double w = (double)(strips * ((ny + seg - 1) / seg)) / (double)slots;
-    const double cost = (w + 0.5 * (std::ceil(w) - w)) * (seg + 2);
-    if (seg == LY || cost < best) best = cost, pick = seg;  // ties keep the longer segment
-  }
-  return pick;
-}
-
-// Segment rows of the Allen-Cahn TMA step (with or without obstacles).  The
-// 16-bit deviation step is bound by instruction issue, so blocks of a
-// partial wave run faster and one wave of blocks suffices; FP64 keeps the
-// two-wave rule.
+// Segment rows of the 16-bit Allen-Cahn TMA step (with or without
+// obstacles): it is bound by instruction issue, so blocks of a partial wave
+// run faster and one wave of blocks suffices.
 template <class C>
 static int tma_segment_rows(int nx, int ny) {
   using G = TmaCfg<C>;
-  const int per_sm = G::threads / G::TBX;
-  if (C::dev) return segment_rows(nx, ny, G::TBX, per_sm, 1);
-  if (G::fp32) return segment_rows_waves(nx, ny, G::TBX, per_sm);
-  return segment_rows(nx, ny, G::TBX, per_sm);
+  return segment_rows(nx, ny, G::TBX, G::threads / G::TBX, 1);
 }
 
 // Launch `kern` as a programmatic dependent of the kernel launched just
@@ -109,11 +84,85 @@ static cudaError_t launch_maybe_dependent(bool dependent, void (*kern)(KArgs...)
   return cudaLaunchKernelEx(&cfg, kern, args...);
 }
 
+// Tile of the one-node-per-thread pass; columns in equal strips of at most 32.
+// FP32: 32 x 4 (4096^2: 522 us a step; 32 x 8 564); Cahn-Hilliard, whose ring is
+// two nodes wide: 32 x 8.  FP64: 32 x 8, and on grids of
+// few nodes 16 x 4 or 8 x 4, so that as many SMs as possible get nodes for
+// their FP64 pipes (300 x 150: 26.7 us; 32 x 8 33.1).
+template <class C>
+static dim3 tile_shape(int nx, int ny, bool ch) {
+  const bool fp64 = sizeof(typename C::value_t) == 8;
+  const long long nodes = (long long)nx * ny, sms = device_sm_count();
+  int t = fp64 ? (nodes < (1LL << 17) ? 64 : 256) : (ch ? 256 : 128);
+  if (fp64 && nodes <= 64 * sms) t = 32;
+  const int wide = t >= 128 ? 32 : (t == 64 ? 16 : 8);
+  const int strips = (nx + wide - 1) / wide, bw = (nx + strips - 1) / strips;
+  return dim3(bw, std::max(1, std::min(t / bw, ny)));
+}
+
+template <class C, int MODEL, int MODE, bool UR, bool OBS = false, bool MOM = sizeof(typename C::value_t) == 4>
+static cudaError_t launch_tile_kernel(const Phys<typename C::value_t>& P, const Bufs<typename C::value_t>& B,
+                                      cudaStream_t s) {
+  using T = typename C::value_t;
+  const dim3 b = tile_shape<C>(P.nx, P.ny, MODEL == MODEL_CH);
+  constexpr int R = MODEL == MODEL_CH || OBS ? 2 : 1;
+  size_t smem = sizeof(T) * (b.x + 2 * R) * (b.y + 2 * R);
+  if (MODEL == MODEL_CH) smem += sizeof(T) * (b.x + 2) * (b.y + 2);
+  const dim3 grid((P.nx + b.x - 1) / b.x, (P.ny + b.y - 1) / b.y);
+  // A dependent launch places its blocks while the kernel before it still holds
+  // SMs, and fills the idle ones unevenly.  FP64 blocks, which keep their SM's
+  // pipe busy, then share SMs that others could relieve (128^2: 27 us a step
+  // against 14.4), unless a block is one warp and every SM can take one.
+  const bool dep = sizeof(T) == 4 || (b.x * b.y <= 32 && (long long)grid.x * grid.y <= device_sm_count());
+  return launch_maybe_dependent(dep, k_tile<C, MODEL, MODE, UR, OBS, MOM>, grid, b, smem, s, P, B);
+}
+
+// FP64 Allen-Cahn runs with n_delta below its default keep the node update's
+// moment form, operation for operation: the scheme amplifies rounding there (a
+// one-ulp change of phi grows to 3e-3 in 2000 steps at n_delta = 3e-3, to 1e-14
+// at the default 5e-3), so any other order of operations is another trajectory.
+// Narrow channels relax all moments (UR = false), as they always have.
+template <class C>
+static cudaError_t launch_tile_moments(int mode, const Phys<typename C::value_t>& P,
+                                       const Bufs<typename C::value_t>& B, bool unit_rates, cudaStream_t s) {
+  switch (mode) {
+    case MODE_STEP:
+      return unit_rates && P.nx >= 4 * XPAD ? launch_tile_kernel<C, MODEL_AC, MODE_STEP, true, false, true>(P, B, s)
+                                            : launch_tile_kernel<C, MODEL_AC, MODE_STEP, false, false, true>(P, B, s);
+    case MODE_MACRO: return launch_tile_kernel<C, MODEL_AC, MODE_MACRO, false, false, true>(P, B, s);
+    case MODE_HIST: return launch_tile_kernel<C, MODEL_AC, MODE_HIST, false, false, true>(P, B, s);
+    case MODE_INIT: return launch_tile_kernel<C, MODEL_AC, MODE_INIT, false, false, true>(P, B, s);
+    default: return cudaErrorInvalidValue;
+  }
+}
+
+template <class C, int MODEL>
+static cudaError_t launch_tile_model(int mode, const Phys<typename C::value_t>& P,
+                                     const Bufs<typename C::value_t>& B, bool unit_rates, cudaStream_t s) {
+  switch (mode) {
+    case MODE_STEP:
+      return unit_rates ? launch_tile_kernel<C, MODEL, MODE_STEP, true>(P, B, s)
+                        : launch_tile_kernel<C, MODEL, MODE_STEP, false>(P, B, s);
+    case MODE_MACRO: return launch_tile_kernel<C, MODEL, MODE_MACRO, false>(P, B, s);
+    case MODE_HIST: return launch_tile_kernel<C, MODEL, MODE_HIST, false>(P, B, s);
+    case MODE_INIT: return launch_tile_kernel<C, MODEL, MODE_INIT, false>(P, B, s);
+    default: return cudaErrorInvalidValue;
+  }
+}
+template <class C>
+cudaError_t launch_tile(int model, int mode, const Phys<typename C::value_t>& P,
+                        const Bufs<typename C::value_t>& B, bool unit_rates, bool moments, cudaStream_t s) {
+  if constexpr (sizeof(typename C::value_t) == 8)
+    if (moments && model == MODEL_AC) return launch_tile_moments<C>(mode, P, B, unit_rates, s);
+  return model == MODEL_CH ? launch_tile_model<C, MODEL_CH>(mode, P, B, unit_rates, s)
+                           : launch_tile_model<C, MODEL_AC>(mode, P, B, unit_rates, s);
+}
+
 template <class C, bool UR, bool VSEG, bool OBS = false>
 static cudaError_t launch_tma_seg(const Phys<typename C::value_t>& P, const Bufs<typename C::value_t>& B,
                                   int* err, cudaStream_t s, bool dependent = false) {
   using G = TmaCfg<C>;
-  using L = TmaLayout<C, G::TBX, G::DF, G::DG, G::slim>;
+  using L = TmaLayout<C, G::TBX, G::DF, G::DG>;
   // per function and device; cheap next to a step
   cudaError_t e = cudaFuncSetAttribute(k_step_tma<C, UR, VSEG, OBS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)L::bytes);
@@ -139,20 +188,22 @@ static cudaError_t launch_tma_variant(const Phys<typename C::value_t>& P0, const
                           : launch_tma_seg<C, UR, true, OBS>(P, B, err, s, dependent);
 }
 
-// Launch grid of the Allen-Cahn TMA step (strip width, rows per segment).
-template <class C>
-void tma_step_grid(int nx, int ny, int* tbx, int* seg_rows) {
-  *tbx = TmaCfg<C>::TBX;
-  *seg_rows = tma_segment_rows<C>(nx, ny);
-}
-
-// Launch grid of the Cahn-Hilliard TMA step.
+// Launch grid of the step with obstacles: columns and rows of a block.
 template <class C>
 static int tma_ch_segment_rows(int nx, int ny);
 template <class C>
-void tma_ch_step_grid(int nx, int ny, int* tbx, int* seg_rows) {
-  *tbx = TmaChCfg<C>::TBX;
-  *seg_rows = tma_ch_segment_rows<C>(nx, ny);
+void obs_step_grid(int nx, int ny, bool ch, int* bw, int* bh) {
+  if (ch) {
+    *bw = TmaChCfg<C>::TBX;
+    *bh = tma_ch_segment_rows<C>(nx, ny);
+  } else if constexpr (C::dev) {
+    *bw = TmaCfg<C>::TBX;
+    *bh = tma_segment_rows<C>(nx, ny);
+  } else {
+    const dim3 b = tile_shape<C>(nx, ny, false);
+    *bw = b.x;
+    *bh = b.y;
+  }
 }
 
 // Cahn-Hilliard step: same segment rule, its own launch shape (TmaChCfg).
@@ -281,7 +332,7 @@ static cudaError_t obs_model(int mode, const Phys<typename C::value_t>& P, const
   }
 }
 
-// Allen-Cahn step with obstacles on the TMA kernel: phi and its fill over
+// 16-bit Allen-Cahn step with obstacles on the TMA kernel: phi and its fill over
 // the region the blocks near obstacles read (P.obs_box; the whole grid
 // without P.obs_near), then k_step_tma<..., OBS>, whose near blocks read phi
 // from the plane and the others run the plain step's path.
@@ -358,8 +409,13 @@ cudaError_t launch_obs(int model, int mode, const Phys<typename C::value_t>& P, 
                        typename C::value_t* phis, typename C::value_t* mus, bool unit_rates, int* err,
                        bool use_tma, cudaStream_t s) {
   if (!P.obs || !phis || (model == MODEL_CH && !mus)) return cudaErrorInvalidValue;
-  if (use_tma && model == MODEL_AC && mode == MODE_STEP && P.nx >= 4 * XPAD)
-    return obs_step_tma<C>(P, B, phis, err, unit_rates, s);
+  if (use_tma && model == MODEL_AC && mode == MODE_STEP && P.nx >= 4 * XPAD) {
+    if constexpr (C::dev) return obs_step_tma<C>(P, B, phis, err, unit_rates, s);
+    else if (!P.obs_near) return cudaErrorInvalidValue;
+    else
+      return unit_rates ? launch_tile_kernel<C, MODEL_AC, MODE_STEP, true, true>(P, B, s)
+                        : launch_tile_kernel<C, MODEL_AC, MODE_STEP, false, true>(P, B, s);
+  }
   if (use_tma && model == MODEL_CH && mode == MODE_STEP && P.nx >= 4 * XPAD)
     return obs_step_tma_ch<C>(P, B, phis, mus, err, unit_rates, s);
   return model == MODEL_CH ? obs_model<C, MODEL_CH>(mode, P, B, phis, mus, unit_rates, s)
@@ -414,17 +470,16 @@ cudaError_t launch_adjoint_init(const Phys<T>& P, const AdjBufs& A, double* out,
 #define PFLBM_INSTANTIATE_CODEC(C)                                                                  \
   template cudaError_t launch_march<C>(int, int, const Phys<C::value_t>&, const Bufs<C::value_t>&,  \
                                        cudaStream_t);                                               \
+  template cudaError_t launch_obs<C>(int, int, const Phys<C::value_t>&, const Bufs<C::value_t>&,    \
+                                     C::value_t*, C::value_t*, bool, int*, bool, cudaStream_t);     \
+  template void obs_step_grid<C>(int, int, bool, int*, int*);
+
+#define PFLBM_INSTANTIATE_DEV(C)                                                                    \
+  PFLBM_INSTANTIATE_CODEC(C)                                                                        \
   template cudaError_t launch_step_tma<C>(const Phys<C::value_t>&, const Bufs<C::value_t>&, int*,   \
                                           bool, cudaStream_t);                                      \
   template cudaError_t launch_step_tma_ch<C>(const Phys<C::value_t>&, const Bufs<C::value_t>&, int*, \
                                              bool, cudaStream_t);                                   \
-  template cudaError_t launch_obs<C>(int, int, const Phys<C::value_t>&, const Bufs<C::value_t>&,    \
-                                     C::value_t*, C::value_t*, bool, int*, bool, cudaStream_t);     \
-  template void tma_step_grid<C>(int, int, int*, int*);                                               \
-  template void tma_ch_step_grid<C>(int, int, int*, int*);
-
-#define PFLBM_INSTANTIATE_DEV(C)                                                                    \
-  PFLBM_INSTANTIATE_CODEC(C)                                                                        \
   template cudaError_t launch_pull_export<C>(const Phys<C::value_t>&, const void*, int, int, double*, \
                                              double, int, int, int, int, cudaStream_t);             \
   template cudaError_t launch_restream<C>(const Phys<C::value_t>&, const C::value_t*, void*, int,   \
@@ -433,6 +488,8 @@ cudaError_t launch_adjoint_init(const Phys<T>& P, const AdjBufs& A, double* out,
 // the arithmetic-type wrappers
 #define PFLBM_INSTANTIATE(T)                                                                        \
   PFLBM_INSTANTIATE_CODEC(PopPlain<T>)                                                              \
+  template cudaError_t launch_tile<PopPlain<T>>(int, int, const Phys<T>&, const Bufs<T>&, bool, bool, \
+                                                cudaStream_t);                                     \
   template cudaError_t launch_pull<T>(const Phys<T>&, const T*, T*, cudaStream_t);                \
   template cudaError_t launch_unstream<T>(const Phys<T>&, const T*, T*, cudaStream_t);            \
   template cudaError_t launch_export<T>(const Phys<T>&, const T*, int, int, double*, double, int,  \

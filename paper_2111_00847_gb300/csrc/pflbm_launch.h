@@ -17,21 +17,23 @@ namespace pflbm {
 template <class C>
 cudaError_t launch_march(int model, int mode, const Phys<typename C::value_t>& P,
                          const Bufs<typename C::value_t>& B, cudaStream_t s);
-// TMA-staged Allen-Cahn step (returns cudaErrorNotSupported when the grid is
-// too narrow for it; the caller then uses launch_march)
+// a pass (any mode) of the plain codecs, one node per thread; moments: keep the
+// FP64 update's moment form
+template <class C>
+cudaError_t launch_tile(int model, int mode, const Phys<typename C::value_t>& P,
+                        const Bufs<typename C::value_t>& B, bool unit_rates, bool moments, cudaStream_t s);
+// TMA-staged steps of the 16-bit deviation codecs (they return
+// cudaErrorNotSupported when the grid is too narrow; the caller then uses
+// launch_march)
 template <class C>
 cudaError_t launch_step_tma(const Phys<typename C::value_t>& P, const Bufs<typename C::value_t>& B, int* err,
                             bool unit_rates, cudaStream_t s);
-// its launch grid: strip width and rows per segment on the current device
-template <class C>
-void tma_step_grid(int nx, int ny, int* tbx, int* seg_rows);
-// the Cahn-Hilliard step's launch grid
-template <class C>
-void tma_ch_step_grid(int nx, int ny, int* tbx, int* seg_rows);
-// TMA-staged Cahn-Hilliard step (the same contract)
 template <class C>
 cudaError_t launch_step_tma_ch(const Phys<typename C::value_t>& P, const Bufs<typename C::value_t>& B, int* err,
                                bool unit_rates, cudaStream_t s);
+// columns and rows of a block of the step with obstacles on the current device
+template <class C>
+void obs_step_grid(int nx, int ny, bool ch, int* bw, int* bh);
 // deviation storage: pulled plane k of a set -> dense doubles of a region
 template <class C>
 cudaError_t launch_pull_export(const Phys<typename C::value_t>& P, const void* in, int set, int k, double* out,
@@ -57,8 +59,8 @@ cudaError_t launch_diag(const Phys<T>& P, const T* macro, const T* phi_prev, dou
 // solid obstacles (pflbm_obstacle.cuh): the reflecting links of every node
 // from a dense byte mask, and one step (or MACRO / HIST / INIT pass) through
 // the obstacle passes; phis, mus: one-plane work planes of the arithmetic
-// type.  With use_tma the Allen-Cahn step runs its node update on the TMA
-// kernel (err: its time-out flag).
+// type.  With use_tma the step runs on the tile (Allen-Cahn, plain storage) or
+// TMA kernels (err: their time-out flag).
 template <typename T>
 cudaError_t launch_obs_links(const Phys<T>& P, const unsigned char* solid, uint16_t* obs, cudaStream_t s);
 template <class C>

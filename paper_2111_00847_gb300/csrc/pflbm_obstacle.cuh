@@ -19,15 +19,17 @@
 //               -> phi plane
 //   k_obs_mu    (CH) mu_phi of Eq. (5) at fluid nodes -> mu plane, then
 //   k_obs_fill  its neutral-wetting values
-// The step's node update then runs on the TMA step kernels instantiated with
-// OBS (pflbm_kernels.cuh).  There only the blocks near an obstacle read the
-// planes (the others run the plain step's path), so per step the passes
-// cover only the regions those blocks read.  k_obs_node is the same update
-// one thread per node: the initial state, history and macroscopic passes,
-// and the step under LBM_FLAG_NO_TMA or on grids under 16 columns, with the
-// passes over whole planes.  It takes the stencils from the planes with the
-// wall ghosts of Eq. (50) (mirror for mu_phi), pulls with reflection at
-// solid links, collides and stores.
+// The 16-bit and Cahn-Hilliard steps then run the node update on the TMA step
+// kernels instantiated with OBS (pflbm_kernels.cuh), where only the blocks near
+// an obstacle read the planes (the others run the plain step's path), so per
+// step the passes cover only the regions those blocks read.  The FP32 and FP64
+// Allen-Cahn step needs none of this: a near block of k_tile forms phi and its
+// fill in shared memory (tile_near_obstacle).  k_obs_node is the same update one
+// thread per node: the initial state, history and macroscopic passes, and the
+// step under LBM_FLAG_NO_TMA or on grids under 16 columns, with the passes over
+// whole planes.  It takes the stencils from the planes with the wall ghosts of
+// Eq. (50) (mirror for mu_phi), pulls with reflection at solid links, collides
+// and stores.
 #pragma once
 
 #include "pflbm_kernels.cuh"
@@ -225,10 +227,8 @@ __global__ void k_obs_mu(const Phys<T> P, const T* __restrict__ phis, T* __restr
   if ((P.obs[(long long)y * P.nx + x] >> OBS_SOLID) & 1u) return;  // filled by k_obs_fill
   T p[9];
   obs_gather9(P, phis, x, y, true, p);
-  const T ph = p[0];
-  const T lap = (((p[1] - ph) + (p[3] - ph)) + ((p[2] - ph) + (p[4] - ph))) * T(2.0 / 3.0) +
-                (((p[5] - ph) + (p[7] - ph)) + ((p[6] - ph) + (p[8] - ph))) * T(1.0 / 6.0);
-  mus[ix(P, 1, 0, x, y)] = P.beta4 * (ph - P.phiA) * (ph - P.phiB) * (ph - P.phibar) - P.kappa * lap;
+  const T pm[3] = {p[7], p[4], p[8]}, p0[3] = {p[3], p[0], p[1]}, pp[3] = {p[6], p[2], p[5]};
+  mus[ix(P, 1, 0, x, y)] = chem_pot_rows<PopPlain<T>>(P, pm + 1, p0 + 1, pp + 1);
 }
 
 // Node update of every node in a mode; solid nodes write zeros.  One node
@@ -285,7 +285,7 @@ __global__ void __launch_bounds__(OBS_THREADS, 8) k_obs_node(const Phys<typename
       for (int k = 0; k < 5; ++k) h[k] = B.hist[ix(P, 5, k, x, y)];
     }
   }
-  node_update<C, MODEL, MODE, UR>(P, B, x, y, phi9, mu9, f, g, h, uin, vin, pin);
+  node_update_nine<C, MODEL, MODE, UR>(P, NodeSink<C, MODE>{P, B, x, y}, phi9, mu9, f, g, h, uin, vin, pin);
 }
 
 }  // namespace pflbm
