@@ -496,6 +496,8 @@ __global__ void k_adj_gather(const Phys<T> P, const T* __restrict__ lp9, T* __re
 // Ghost rows beyond y walls, over the extended x range (one thread a column).
 template <typename T>
 __global__ void k_adj_fold_y(const Phys<T> P, const T* __restrict__ phi, T* __restrict__ lext) {
+  asm volatile("griddepcontrol.launch_dependents;");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   const int x = (int)(blockIdx.x * blockDim.x + threadIdx.x) - P.wall_x;
   if (x >= P.nx + P.wall_x || !P.wall_y) return;
   T d1, d2;
@@ -512,6 +514,8 @@ __global__ void k_adj_fold_y(const Phys<T> P, const T* __restrict__ phi, T* __re
 // Ghost columns beyond x walls (one thread a row).
 template <typename T>
 __global__ void k_adj_fold_x(const Phys<T> P, const T* __restrict__ phi, T* __restrict__ lext) {
+  asm volatile("griddepcontrol.launch_dependents;");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   const int y = blockIdx.x * blockDim.x + threadIdx.x;
   if (y >= P.ny || !P.wall_x) return;
   T d1, d2;
@@ -590,6 +594,8 @@ __global__ void k_adj_init(const Phys<T> P, const T* __restrict__ lf, const T* _
 // Sum of the per-block dJ/dG partials into acc[2].
 template <typename T>
 __global__ void k_adj_reduce(const double* __restrict__ part, long long nparts, double* __restrict__ acc) {
+  asm volatile("griddepcontrol.launch_dependents;");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   __shared__ double red[256 / 32][2];
   double sx = 0.0, sy = 0.0;
   for (long long b = threadIdx.x; b < nparts; b += blockDim.x) {
@@ -618,5 +624,360 @@ __global__ void k_adj_reduce(const double* __restrict__ part, long long nparts, 
   }
 }
 
-}  // namespace pflbm
 
+// ---------------------------------------------------------------------------
+// The adjoint step at unit rates (the rates the paper leaves at 1 are 1).
+//
+// The adjoints of a node's pulled populations then span few directions, so the
+// node pass hands over 14 values per node instead of 27: the adjoint of phi,
+// lap phi and grad phi (4, from which any stencil value's adjoint follows), of
+// f's first moments (2), and of g through p, the moments 3..8 (8: see below).
+// k_adj_tile forms phi of a tile in shared memory (no pass for it) and sweeps
+// the node update backwards in the form of node_update; k_adj_gather4 applies
+// the transposed stencils, the folds are the ones above, and k_adj_stream14
+// builds the adjoint of the post-collision populations.  Per node and step 43
+// values in and 19 out, 4 and 1, 15 and 18 against 136 in all before.
+// In FP64 the pass is bound by the FP64 pipe: about 300 operations a node in
+// k_adj_tile, 640 in k_adj_node (512 x 2048: 1230 us in k_adj_node alone, 830 us
+// for all passes now; with 128 registers and 16 warps per SM, which spill 40
+// bytes, 8 % less time than with 150 and 8).  FP32 waits on memory: 500 x 1000
+// 110 us a step in all passes, 60 now.  Whole gradients, forward and
+// recomputation included: 512 x 2048 FP64 20 steps 47.7 -> 34.7 ms, 500 x 1000
+// FP32 40 steps 7.5 -> 6.2 ms.
+// ---------------------------------------------------------------------------
+constexpr int ADJ4 = 4;  // planes: phi, lap phi, d/dx, d/dy
+constexpr int ADJF = 2;  // f: moments 3, 5
+// g: q/0.6 +- moment 7 (axes x, y), q +- moment 8 (diagonals 5/7, 6/8), then the
+// first-order parts of the axes (x, y) and of the diagonals (x, y)
+constexpr int ADJG = 8;
+
+template <typename T>
+__device__ __forceinline__ void node_adjoint_unit(const Phys<T>& P, const Row3<T> fr[3], const T g[9], T h3, T h4,
+                                                  const T lfs[9], const T lgs[9], const T lhn[5], T o4[ADJ4],
+                                                  T of[ADJF], T og[ADJG], T lh[5], T& lGx, T& lGy) {
+  // ---- forward: the quantities of node_update that the sweep needs
+  const T phi = fr[1].c;
+  const T gx = grad_x(fr[0], fr[1], fr[2]), gy = grad_y(fr[0], fr[2]);
+  const T pa = sb(phi, P.phiA), pb = sb(phi, P.phiB), pc = sb(phi, P.phibar);
+  const T pab = ml(pa, pb), bpc = ml(P.beta4, pc);
+  const T mu = fm(bpc, pab, ml(-P.kappa, laplace(fr[0], fr[1], fr[2])));
+  const T g2 = fm(gx, gx, ml(gy, gy));
+  const T inv = inv_root4(fm(g2, g2, P.n_delta4));
+  const T linv_ = ml(P.lam_coef, inv);  // d li / d pab
+  const T li = ml(linv_, pab);
+  const T cm = fm(-P.mob_drho, li, -P.mob_drho);
+  const T rho = fm(P.drho, pb, P.rhoB);
+  const T Gs = P.gravity_mode == 0 ? T(1) : (P.gravity_mode == 1 ? rho : sb(rho, P.rho_mean));
+  const T Fx = fm(mu, gx, ml(Gs, P.gx)), Fy = fm(mu, gy, ml(Gs, P.gy));
+  const Pairs<T> pg = pairs_of(g);
+  const T irho = recip(rho);
+  const T E3 = fm(T(0.5), Fx, ad(pg.d13, pg.gx)), E5 = fm(T(0.5), Fy, ad(pg.d24, pg.gy));
+  const T u = ml(E3, irho), v = ml(E5, irho);
+  const T vgy = ml(v, gy);
+  const T ug = fm(u, gx, vgy), ugm = fm(u, gx, -vgy), ugx = fm(u, gy, ml(v, gx));
+  const T cA = ml(cm, ugm), cB = ml(cm, ugx);
+  T s7 = P.sg[7], s8 = P.sg[8], dsn = T(0);  // viscous rates, d snode / d phi
+  if (P.sg7_node | P.sg8_node) {
+    const T num = P.visc_inverse ? fm(P.c_num1, pb, P.c_num0) : rho;
+    const T rd = recip(fm(P.c_den1, pb, P.c_den0));
+    const T snode = ml(num, rd);
+    dsn = ml(fm(-P.c_den1, snode, P.c_num1), rd);
+    if (P.sg7_node) s7 = snode;
+    if (P.sg8_node) s8 = snode;
+  }
+
+  // ---- f collision
+  const Pairs<T> pf = pairs_of(lfs);
+  T lphi = fm(P.c_eta9, fm(T(0.25), ad(pf.s57, pf.s68), fm(T(-5), lfs[0], ad(pf.s13, pf.s24))), lfs[0]);
+  const T fjx = ad(pf.d13, pf.gx), frx = fm(T(-2), pf.d13, pf.gx);
+  const T fjy = ad(pf.d24, pf.gy), fry = fm(T(-2), pf.d24, pf.gy);
+  of[0] = ml(P.c_fa[0][0], fjx);
+  of[1] = ml(P.c_fa[1][0], fjy);
+  T lphu = fm(P.c_fa[0][1], fjx, ml(T(-1.0 / 12.0), frx)), lphv = fm(P.c_fa[1][1], fjy, ml(T(-1.0 / 12.0), fry));
+  const T lXx = fm(P.c_fa[0][2], fjx, ml(T(-1.0 / 24.0), frx));
+  const T lXy = fm(P.c_fa[1][2], fjy, ml(T(-1.0 / 24.0), fry));
+
+  // ---- g collision
+  const Pairs<T> pl = pairs_of(lgs);
+  const T sa = ad(pl.s13, pl.s24), sd = ad(pl.s57, pl.s68);
+  const T x12 = ml(T(1.0 / 12.0), ad(sa, sd));
+  const T lq = fm(T(0.05), sd, fm(T(0.2), sa, -lgs[0]));
+  const T lw = fm(T(-2.0 / 3.0), lgs[0], x12);
+  const T gjx = ad(pl.d13, pl.gx), grx = fm(T(-2), pl.d13, pl.gx);
+  const T gjy = ad(pl.d24, pl.gy), gry = fm(T(-2), pl.d24, pl.gy);
+  T lE3 = fm(P.c_gn[0][0], grx, ml(T(1.0 / 6.0), gjx)), lE5 = fm(P.c_gn[1][0], gry, ml(T(1.0 / 6.0), gjy));
+  T lFx = fm(P.c_gn[0][2], grx, ml(T(1.0 / 12.0), gjx)), lFy = fm(P.c_gn[1][2], gry, ml(T(1.0 / 12.0), gjy));
+  const T lm4 = ml(P.c_gn[0][1], grx), lm6 = ml(P.c_gn[1][1], gry);
+  const T n7 = ml(T(0.25), sb(pl.s13, pl.s24)), n8 = ml(T(0.25), sb(pl.s57, pl.s68));
+  const T lE7 = ml(s7, n7), lE8 = ml(s8, n8);
+  const T lm7 = sb(n7, lE7), lm8 = sb(n8, lE8);
+  const T lQ7 = fm(T(-0.5), lE7, n7), lQ8 = fm(T(-0.5), lE8, n8);
+  T lpb = T(0);
+  if (P.sg7_node | P.sg8_node) {  // through the node-dependent rates: d m'/ds = eq - m - src / 2
+    const T vFy = ml(v, Fy);
+    const T uFm = fm(u, Fx, -vFy), uFx = fm(u, Fy, ml(v, Fx));
+    T lsn = T(0);
+    if (P.sg7_node) {
+      const T Q7 = fm(P.c_ug7, ugm, fm(T(2), uFm, sb(cA, h3)));
+      const T E7 = fm(u, E3, fm(-v, E5, cA));
+      lsn = ml(n7, fm(T(-0.5), Q7, sb(E7, sb(pg.s13, pg.s24))));
+    }
+    if (P.sg8_node) {
+      const T Q8 = fm(P.c_ug8, ugx, fm(T(0.5), sb(cB, h4), uFx));
+      const T E8 = fm(u, E5, ml(T(0.5), cB));
+      lsn = fm(n8, fm(T(-0.5), Q8, sb(E8, sb(pg.s57, pg.s68))), lsn);
+    }
+    lpb = ml(lsn, dsn);
+  }
+  // q, Z, t
+  const T lt = fm(P.K, lq, ml(T(0.5), lw));
+  const T lZ = fm(T(-2.0 / 3.0), lq, lw);
+  const T luF = ml(T(2), lt);
+  T lug = fm(P.c_ugq, lq, fm(P.drho, x12, ml(P.c_ug24, sd)));
+  // history outputs and derivatives d = chi - h
+  lh[0] = -lXx;
+  lh[1] = -lXy;
+  lh[2] = -lt;
+  lh[3] = -lQ7;
+  lh[4] = ml(T(-0.5), lQ8);
+  lphu = ad(lphu, ad(lhn[0], lXx));
+  lphv = ad(lphv, ad(lhn[1], lXy));
+  const T lum = ad(ad(lZ, lt), lhn[2]);
+  const T lcA = ad(ad(lE7, lQ7), lhn[3]);
+  const T lcB = fm(T(0.5), ad(lE8, lQ8), lhn[4]);
+  // Z = u E3 + v E5 + um, E7 = u E3 - v E5 + cA, E8 = u E5 + cB / 2
+  const T zp = ad(lZ, lE7), zm = sb(lZ, lE7);
+  T lu = fm(zp, E3, ml(lE8, E5)), lv = ml(zm, E5);
+  lE3 = fm(zp, u, lE3);
+  lE5 = fm(zm, v, fm(lE8, u, lE5));
+  // um, cA, cB = cm (ug, ugm, ugx)
+  const T lcm = fm(lum, ug, fm(lcA, ugm, ml(lcB, ugx)));
+  lug = fm(cm, lum, lug);
+  const T lugm = fm(cm, lcA, ml(P.c_ug7, lQ7));
+  const T lugx = fm(cm, lcB, ml(P.c_ug8, lQ8));
+  // products with F: 2 t, 2 Q7, Q8
+  const T fp = fm(T(2), lQ7, luF), fn = fm(T(-2), lQ7, luF);
+  lu = fm(fp, Fx, fm(lQ8, Fy, lu));
+  lv = fm(fn, Fy, fm(lQ8, Fx, lv));
+  lFx = fm(fp, u, fm(lQ8, v, lFx));
+  lFy = fm(fn, v, fm(lQ8, u, lFy));
+  // products with grad phi
+  const T gp = ad(lug, lugm), gn = sb(lug, lugm);
+  lu = fm(gp, gx, fm(lugx, gy, lu));
+  lv = fm(gn, gy, fm(lugx, gx, lv));
+  T lgx = fm(gp, u, ml(lugx, v)), lgy = fm(gn, v, ml(lugx, u));
+  // phi u, phi v
+  lu = fm(phi, lphu, lu);
+  lv = fm(phi, lphv, lv);
+  lphi = fm(u, lphu, fm(v, lphv, lphi));
+  // u = E3 / rho, E3 = j + F / 2
+  T lrho = ml(-fm(lu, u, ml(lv, v)), irho);
+  lE3 = fm(lu, irho, lE3);
+  lE5 = fm(lv, irho, lE5);
+  lFx = fm(T(0.5), lE3, lFx);
+  lFy = fm(T(0.5), lE5, lFy);
+  og[0] = ad(lq, lm7);
+  og[1] = sb(lq, lm7);
+  og[2] = ad(lq, lm8);
+  og[3] = sb(lq, lm8);
+  og[4] = fm(T(-2), lm4, lE3);
+  og[5] = fm(T(-2), lm6, lE5);
+  og[6] = ad(lm4, lE3);
+  og[7] = ad(lm6, lE5);
+  // F = mu grad phi + Gs G
+  const T lmu = fm(lFx, gx, ml(lFy, gy));
+  lgx = fm(lFx, mu, lgx);
+  lgy = fm(lFy, mu, lgy);
+  lGx = ml(lFx, Gs);
+  lGy = ml(lFy, Gs);
+  if (P.gravity_mode != 0) lrho = fm(lFx, P.gx, fm(lFy, P.gy, lrho));
+  lpb = fm(P.drho, lrho, lpb);
+  // cm = -mob (1 + li), X = d(phi u) - li grad phi / 3
+  const T li3 = ml(T(-1.0 / 3.0), li);
+  const T lli = fm(-P.mob_drho, lcm, ml(T(-1.0 / 3.0), fm(lXx, gx, ml(lXy, gy))));
+  lgx = fm(li3, lXx, lgx);
+  lgy = fm(li3, lXy, lgy);
+  // li = lam_coef pab r, r = (|grad phi|^4 + delta^4)^(-1/4), dr = -|g|^2 r^5 g.dg
+  const T r2 = ml(inv, inv);
+  const T gl = -ml(ml(ml(lli, li), g2), ml(r2, r2));
+  lgx = fm(gx, gl, lgx);
+  lgy = fm(gy, gl, lgy);
+  // mu = beta4 pc pab - kappa lap
+  const T lpab = fm(bpc, lmu, ml(linv_, lli));
+  lpb = fm(pa, lpab, lpb);
+  lphi = ad(ad(lphi, lpb), fm(pb, lpab, ml(ml(P.beta4, pab), lmu)));
+  o4[0] = lphi;
+  o4[1] = ml(-P.kappa, lmu);
+  o4[2] = lgx;
+  o4[3] = lgy;
+}
+
+template <typename T>
+__global__ void __launch_bounds__(TILE_THREADS, 2)
+    k_adj_tile(const Phys<T> P, const T* __restrict__ fin, const T* __restrict__ gin, const T* __restrict__ hist,
+               T* __restrict__ phi, const T* __restrict__ lf, const T* __restrict__ lg, T* __restrict__ lh,
+               T* __restrict__ p4, T* __restrict__ pf, T* __restrict__ pg, double* __restrict__ gpart, int hist_only) {
+  extern __shared__ __align__(16) unsigned char tile_smem[];
+  const int bw = blockDim.x, bh = blockDim.y, pw = bw + 2;
+  T* const sp = reinterpret_cast<T*>(tile_smem);  // [bh + 2][pw]
+  const int tx = threadIdx.x, ty = threadIdx.y;
+  const int tid = ty * bw + tx, nth = bw * bh;
+  const int x0 = blockIdx.x * bw, y0 = blockIdx.y * bh;
+  const int w = min(bw, P.nx - x0), hgt = min(bh, P.ny - y0);
+  const bool active = tx < w && ty < hgt;
+  const int x = x0 + tx, y = y0 + ty;
+  asm volatile("griddepcontrol.launch_dependents;");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  T f[9], g[9], lfs[9], lgs[9], lhn[5], h3 = T(0), h4 = T(0);
+  if (active) {
+    pull9<PopPlain<T>>(fin, P, 0, x, y, f);
+    pull9<PopPlain<T>>(gin, P, 1, x, y, g);
+    const long long i9 = ix(P, 9, 0, x, y), i5 = ix(P, 5, 0, x, y), pc = P.pitch;
+#pragma unroll
+    for (int i = 0; i < 9; ++i) {
+      lfs[i] = hist_only ? T(0) : lf[i9 + i * pc];
+      lgs[i] = hist_only ? T(0) : lg[i9 + i * pc];
+    }
+#pragma unroll
+    for (int k = 0; k < 5; ++k) lhn[k] = lh[i5 + k * pc];
+    if (!hist_only) h3 = hist[i5 + 3 * pc], h4 = hist[i5 + 4 * pc];
+  }
+  Bufs<T> B;
+  B.fin = fin;
+  tile_ring<PopPlain<T>, MODE_STEP, 1>(P, B, sp, pw, x0, y0, w, hgt, tid, nth);
+  if (active) {
+    const T ph = sum9(f);
+    sp[(ty + 1) * pw + tx + 1] = ph;
+    phi[ix(P, 1, 0, x, y)] = ph;  // for the folds of the wetting ghosts
+  }
+  __syncthreads();
+  tile_ghosts<1>(P, sp, pw, x0, y0, w, hgt, tid, nth);
+  T gxs = T(0), gys = T(0);
+  if (active) {
+    const T* const q = sp + (ty + 1) * pw + tx + 1;
+    const Row3<T> fr[3] = {row3_at(q - pw), row3_at(q), row3_at(q + pw)};
+    T o4[ADJ4], of[ADJF], og[ADJG], lho[5];
+    node_adjoint_unit(P, fr, g, h3, h4, lfs, lgs, lhn, o4, of, og, lho, gxs, gys);
+    const long long pc = P.pitch;
+    const long long i4 = ix(P, ADJ4, 0, x, y), i2 = ix(P, ADJF, 0, x, y), i8 = ix(P, ADJG, 0, x, y);
+#pragma unroll
+    for (int k = 0; k < ADJ4; ++k) p4[i4 + k * pc] = o4[k];
+#pragma unroll
+    for (int k = 0; k < ADJF; ++k) pf[i2 + k * pc] = of[k];
+#pragma unroll
+    for (int k = 0; k < ADJG; ++k) pg[i8 + k * pc] = og[k];
+    const long long i5 = ix(P, 5, 0, x, y);
+#pragma unroll
+    for (int k = 0; k < 5; ++k) lh[i5 + k * pc] = lho[k];
+  }
+  // block sums of dJ/dG: over the warps' lanes in the arithmetic type, the rest
+  // in double (one warp's additions instead of every warp's: FP64 ones cost)
+  __shared__ T red[2][TILE_THREADS];
+  red[0][tid] = gxs;
+  red[1][tid] = gys;
+  __syncthreads();
+  if (tid < 32) {
+    T a = T(0), b = T(0);
+    for (int k = tid; k < nth; k += 32) {
+      a += red[0][k];
+      b += red[1][k];
+    }
+    double sx = double(a), sy = double(b);
+    const unsigned mask = __activemask();  // blocks of fewer than 32 threads
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const double ox = __shfl_down_sync(mask, sx, o), oy = __shfl_down_sync(mask, sy, o);
+      if (tid + o < min(nth, 32)) sx += ox, sy += oy;
+    }
+    if (tid == 0) {
+      const long long b = (long long)blockIdx.y * gridDim.x + blockIdx.x;
+      gpart[2 * b] = sx;
+      gpart[2 * b + 1] = sy;
+    }
+  }
+}
+
+// k_adj_gather from the adjoints of phi, lap phi and grad phi: the transposed
+// stencils.
+template <typename T>
+__global__ void k_adj_gather4(const Phys<T> P, const T* __restrict__ p4, T* __restrict__ lext) {
+  asm volatile("griddepcontrol.launch_dependents;");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  const int x = (int)(blockIdx.x * blockDim.x + threadIdx.x) - P.wall_x;
+  const int y = (int)blockIdx.y - P.wall_y;
+  if (x >= P.nx + P.wall_x) return;
+  constexpr int cx[9] = {0, 1, 0, -1, 0, 1, -1, -1, 1};
+  constexpr int cy[9] = {0, 0, 1, 0, -1, 1, 1, -1, -1};
+  const long long pc = P.pitch;
+  T s = T(0), l4 = T(0), l8 = T(0), g4 = T(0), g8 = T(0);
+#pragma unroll
+  for (int k = 0; k < 9; ++k) {
+    int sx = x - cx[k], sy = y - cy[k];  // the node whose stencil point k is (x, y)
+    if (sx < 0 || sx >= P.nx) {
+      if (P.wall_x) continue;
+      sx = sx < 0 ? sx + P.nx : sx - P.nx;
+    }
+    if (sy < 0 || sy >= P.ny) {
+      if (P.wall_y) continue;
+      sy = sy < 0 ? sy + P.ny : sy - P.ny;
+    }
+    const T* const q = p4 + ix(P, ADJ4, 0, sx, sy);
+    if (k == 0) {
+      s = fm(T(-10.0 / 3.0), q[pc], q[0]);
+    } else {
+      const T gg = cy[k] == 0 ? (cx[k] > 0 ? q[2 * pc] : -q[2 * pc])
+                              : (cx[k] == 0 ? (cy[k] > 0 ? q[3 * pc] : -q[3 * pc])
+                                            : ad(cx[k] > 0 ? q[2 * pc] : -q[2 * pc], cy[k] > 0 ? q[3 * pc] : -q[3 * pc]));
+      if (k < 5) l4 = ad(l4, q[pc]), g4 = ad(g4, gg);
+      else l8 = ad(l8, q[pc]), g8 = ad(g8, gg);
+    }
+  }
+  s = fm(T(2.0 / 3.0), l4, fm(T(1.0 / 6.0), l8, s));
+  lext[ext_index(P.nx, x, y)] = fm(T(1.0 / 3.0), g4, fm(T(1.0 / 12.0), g8, s));
+}
+
+// k_adj_stream from the 10 values per node of k_adj_tile and lext.
+template <typename T>
+__global__ void k_adj_stream14(const Phys<T> P, const T* __restrict__ pf, const T* __restrict__ pg,
+                               const T* __restrict__ lext, T* __restrict__ lf, T* __restrict__ lg) {
+  asm volatile("griddepcontrol.launch_dependents;");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y;
+  if (x >= P.nx) return;
+  constexpr int cx[9] = {0, 1, 0, -1, 0, 1, -1, -1, 1};
+  constexpr int cy[9] = {0, 0, 1, 0, -1, 1, 1, -1, -1};
+  const long long pc = P.pitch, i9 = ix(P, 9, 0, x, y);
+  lf[i9] = lext[ext_index(P.nx, x, y)];
+  lg[i9] = T(0);
+#pragma unroll
+  for (int j = 1; j < 9; ++j) {
+    int tx = x + cx[j], ty = y + cy[j];
+    bool wall = false;
+    if (tx < 0 || tx >= P.nx) { if (P.wall_x) wall = true; else tx = tx < 0 ? tx + P.nx : tx - P.nx; }
+    if (ty < 0 || ty >= P.ny) { if (P.wall_y) wall = true; else ty = ty < 0 ? ty + P.ny : ty - P.ny; }
+    // beyond a wall: what the node itself pulled in direction opp(j)
+    const int rx = wall ? x : tx, ry = wall ? y : ty;
+    const T* const a = pf + ix(P, ADJF, 0, rx, ry);
+    const T* const b = pg + ix(P, ADJG, 0, rx, ry);
+    const T le = lext[ext_index(P.nx, rx, ry)];
+    T f1, g1, ge;
+    if (j < 5) {
+      const int d = cx[j] == 0;  // axis x, y
+      f1 = a[d * pc];
+      g1 = b[(4 + d) * pc];
+      ge = b[d * pc];
+      if (cx[j] + cy[j] < 0) f1 = -f1, g1 = -g1;
+    } else {
+      const T fx = a[0], fy = a[pc], gx = b[6 * pc], gy = b[7 * pc];
+      f1 = cx[j] == cy[j] ? ad(fx, fy) : sb(fx, fy);
+      g1 = cx[j] == cy[j] ? ad(gx, gy) : sb(gx, gy);
+      ge = b[(cx[j] == cy[j] ? 2 : 3) * pc];
+      if (cx[j] < 0) f1 = -f1, g1 = -g1;
+    }
+    if (wall) f1 = -f1, g1 = -g1;
+    lf[i9 + j * pc] = ad(le, f1);
+    lg[i9 + j * pc] = ad(ge, g1);
+  }
+}
+
+}  // namespace pflbm

@@ -1052,7 +1052,7 @@ static int ensure_adjoint(lbm_handle* h) {
   const size_t pl = (size_t)h->plane * h->esize;
   void* planes = dev_alloc(h, 51 * pl);  // lf 9, lg 9, lh 5, lp9 9, lfp 9, lgp 9, phi 1
   void* lext = dev_alloc(h, (size_t)(h->nx + 2) * (h->ny + 2) * h->esize);
-  const long long nblocks = (long long)((h->nx + ADJ_THREADS - 1) / ADJ_THREADS) * h->ny;
+  const long long nblocks = h->prec == LBM_FP64 ? adjoint_blocks<double>(h->nx, h->ny) : adjoint_blocks<float>(h->nx, h->ny);
   double* gpart = (double*)dev_alloc(h, (size_t)(2 * nblocks) * sizeof(double));
   double* gacc = (double*)dev_alloc(h, 2 * sizeof(double));
   if (!planes || !lext || !gpart || !gacc) {
@@ -1101,7 +1101,7 @@ static int do_adjoint_seed(lbm_handle* h, const double* djdphi) {
 template <typename T>
 static int do_adjoint_step(lbm_handle* h, const void* state) {
   const Phys<T> P = make_phys<T>(h);
-  CUDA_TRY(h, launch_adjoint_step<T>(P, state, h->pop_bytes, h->adj, h->gacc, false, h->stream));
+  CUDA_TRY(h, launch_adjoint_step<T>(P, state, h->pop_bytes, h->adj, h->gacc, false, h->unit_rates, h->stream));
   return LBM_OK;
 }
 
@@ -1110,7 +1110,7 @@ static int do_adjoint_init(lbm_handle* h, const void* state0, double* out) {
   const Phys<T> P = make_phys<T>(h);
   int rc = ensure_stage(h, 1);
   if (rc) return rc;
-  CUDA_TRY(h, launch_adjoint_step<T>(P, state0, h->pop_bytes, h->adj, h->gacc, true, h->stream));
+  CUDA_TRY(h, launch_adjoint_step<T>(P, state0, h->pop_bytes, h->adj, h->gacc, true, h->unit_rates, h->stream));
   CUDA_TRY(h, launch_adjoint_init<T>(P, h->adj, h->dstage, h->stream));
   const long long N = (long long)h->nx * h->ny;
   CUDA_TRY(h, cudaMemcpyAsync(out, h->dstage, N * sizeof(double), cudaMemcpyDeviceToHost, h->stream));

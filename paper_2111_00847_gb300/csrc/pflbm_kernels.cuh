@@ -451,6 +451,16 @@ __device__ __forceinline__ double fm(double a, double b, double c) { return __fm
 __device__ __forceinline__ double ad(double a, double b) { return __dadd_rn(a, b); }
 __device__ __forceinline__ double sb(double a, double b) { return __dsub_rn(a, b); }
 __device__ __forceinline__ double ml(double a, double b) { return __dmul_rn(a, b); }
+// the same in FP32, for code shared by both types (the adjoint)
+__device__ __forceinline__ float fm(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ float ad(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ float sb(float a, float b) { return __fsub_rn(a, b); }
+__device__ __forceinline__ float ml(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ float recip(float a) { return __fdividef(1.0f, a); }
+__device__ __forceinline__ float inv_root4(float S) {
+  const float y = rsqrtf(S);
+  return ml(y, rsqrtf(y));
+}
 
 // 1 / a: the hardware's seed (rcp.approx.ftz.f64; its relative error was
 // measured below 2^-19.9) and one step of the third-order iteration
@@ -1443,6 +1453,62 @@ struct TileSink {
   }
 };
 
+// phi of a tile's halo ring (in the domain, or wrapped): R rows below and above
+// over the widened columns, then R columns on either side.
+template <class C, int MODE, int R, typename T = typename C::value_t>
+__device__ __forceinline__ void tile_ring(const Phys<T>& P, const Bufs<T>& B, T* sp, int pw, int x0, int y0, int w,
+                                          int hgt, int tid, int nth) {
+  const int nx = P.nx, ny = P.ny;
+  const bool wx = P.wall_x != 0, wy = P.wall_y != 0;
+  const int row_cells = R * (w + 2 * R), ring = 2 * row_cells + 2 * R * hgt;
+  for (int k = tid; k < ring; k += nth) {
+    int cx, cy;
+    if (k < 2 * row_cells) {
+      const int r = k / (w + 2 * R);
+      cx = k - r * (w + 2 * R) - R;
+      cy = r < R ? r - R : hgt + (r - R);
+    } else {
+      const int q = k - 2 * row_cells, r = q / (2 * R), c = q - r * 2 * R;
+      cy = r;
+      cx = c < R ? c - R : w + (c - R);
+    }
+    int xx = x0 + cx, yy = y0 + cy;
+    if ((wx && (xx < 0 || xx >= nx)) || (wy && (yy < 0 || yy >= ny))) continue;  // ghosts follow
+    xx = xx < 0 ? xx + nx : (xx >= nx ? xx - nx : xx);
+    yy = yy < 0 ? yy + ny : (yy >= ny ? yy - ny : yy);
+    sp[(cy + R) * pw + cx + R] = phi_at<C, MODE>(P, B, xx, yy);
+  }
+}
+// Wetting ghosts of a phi tile (after a barrier; ends with one where there are
+// any): the column beyond an x wall on every row the tile and its halo hold,
+// then the row beyond a y wall over the widened columns.  cl, cr, rb, rt: their
+// places relative to the tile (block-uniform; a Cahn-Hilliard tile that ends one
+// node short of a wall holds the ghosts too, for mu_phi of the node between).
+template <int R, typename T>
+__device__ __forceinline__ void tile_ghosts(const Phys<T>& P, T* sp, int pw, int x0, int y0, int w, int hgt, int tid,
+                                            int nth) {
+  const bool wx = P.wall_x != 0, wy = P.wall_y != 0;
+  const int cl = -1 - x0, cr = P.nx - x0, rb = -1 - y0, rt = P.ny - y0;
+  const bool has_l = wx && cl >= -R, has_r = wx && cr < w + R;
+  const bool has_b = wy && rb >= -R, has_t = wy && rt < hgt + R;
+  if (has_l || has_r) {
+    for (int r = tid; r < hgt + 2 * R; r += nth) {
+      T* const q = sp + r * pw + R;
+      if (has_l) q[cl] = wall_ghost(P, SIDE_LEFT, q[cl + 1], q[cl + 2]);
+      if (has_r) q[cr] = wall_ghost(P, SIDE_RIGHT, q[cr - 1], q[cr - 2]);
+    }
+    __syncthreads();
+  }
+  if (has_b || has_t) {
+    for (int c = tid; c < w + 2 * R; c += nth) {
+      T* const q = sp + R * pw + c;
+      if (has_b) q[rb * pw] = wall_ghost(P, SIDE_BOTTOM, q[(rb + 1) * pw], q[(rb + 2) * pw]);
+      if (has_t) q[rt * pw] = wall_ghost(P, SIDE_TOP, q[(rt - 1) * pw], q[(rt - 2) * pw]);
+    }
+    __syncthreads();
+  }
+}
+
 // The update of a tile that reaches a solid obstacle (Allen-Cahn STEP; a solid
 // node within 3 nodes of the tile): phi of the fluid nodes up to two nodes out
 // from mask-aware pulls, then the neutral-wetting value at the solid nodes of
@@ -1641,52 +1707,10 @@ __global__ void __launch_bounds__(TILE_THREADS, (TileCfg<typename C::value_t, MO
         }
       }
     }
-    // the halo ring (in the domain, or wrapped): R rows below and above over the
-    // widened columns, then R columns on either side
-    const int row_cells = R * (w + 2 * R), ring = 2 * row_cells + 2 * R * hgt;
-    for (int k = tid; k < ring; k += nth) {
-      int cx, cy;
-      if (k < 2 * row_cells) {
-        const int r = k / (w + 2 * R);
-        cx = k - r * (w + 2 * R) - R;
-        cy = r < R ? r - R : hgt + (r - R);
-      } else {
-        const int q = k - 2 * row_cells, r = q / (2 * R), c = q - r * 2 * R;
-        cy = r;
-        cx = c < R ? c - R : w + (c - R);
-      }
-      int xx = x0 + cx, yy = y0 + cy;
-      if ((wx && (xx < 0 || xx >= nx)) || (wy && (yy < 0 || yy >= ny))) continue;  // ghosts follow
-      xx = xx < 0 ? xx + nx : (xx >= nx ? xx - nx : xx);
-      yy = yy < 0 ? yy + ny : (yy >= ny ? yy - ny : yy);
-      sp[(cy + R) * pw + cx + R] = phi_at<C, MODE>(P, B, xx, yy);
-    }
+    tile_ring<C, MODE, R>(P, B, sp, pw, x0, y0, w, hgt, tid, nth);
     if (active) sp[(ty + R) * pw + tx + R] = MODE == MODE_INIT ? T(B.iphi[(long long)y * nx + x]) : sum9(f);
     __syncthreads();
-    // wetting ghosts: the column beyond an x wall on every row the tile and its
-    // halo hold, then the row beyond a y wall over the widened columns.  cl, cr,
-    // rb, rt: their places relative to the tile (block-uniform; a Cahn-Hilliard
-    // tile that ends one node short of a wall holds the ghosts too, for mu_phi
-    // of the node between)
-    const int cl = -1 - x0, cr = nx - x0, rb = -1 - y0, rt = ny - y0;
-    const bool has_l = wx && cl >= -R, has_r = wx && cr < w + R;
-    const bool has_b = wy && rb >= -R, has_t = wy && rt < hgt + R;
-    if (has_l || has_r) {
-      for (int r = tid; r < hgt + 2 * R; r += nth) {
-        T* const q = sp + r * pw + R;
-        if (has_l) q[cl] = wall_ghost(P, SIDE_LEFT, q[cl + 1], q[cl + 2]);
-        if (has_r) q[cr] = wall_ghost(P, SIDE_RIGHT, q[cr - 1], q[cr - 2]);
-      }
-      __syncthreads();
-    }
-    if (has_b || has_t) {
-      for (int c = tid; c < w + 2 * R; c += nth) {
-        T* const q = sp + R * pw + c;
-        if (has_b) q[rb * pw] = wall_ghost(P, SIDE_BOTTOM, q[(rb + 1) * pw], q[(rb + 2) * pw]);
-        if (has_t) q[rt * pw] = wall_ghost(P, SIDE_TOP, q[(rt - 1) * pw], q[(rt - 2) * pw]);
-      }
-      __syncthreads();
-    }
+    tile_ghosts<R>(P, sp, pw, x0, y0, w, hgt, tid, nth);
   }
   if (MODEL == MODEL_CH) {
     // mu_phi on the tile and one node around it; beyond walls the mirror value

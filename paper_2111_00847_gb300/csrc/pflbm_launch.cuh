@@ -422,33 +422,65 @@ cudaError_t launch_obs(int model, int mode, const Phys<typename C::value_t>& P, 
                            : obs_model<C, MODEL_AC>(mode, P, B, phis, mus, unit_rates, s);
 }
 
+// Blocks of an adjoint node pass (each leaves a pair of dJ/dG partial sums).
+template <typename T>
+long long adjoint_blocks(int nx, int ny) {
+  const dim3 b = tile_shape<PopPlain<T>>(nx, ny, false);
+  return std::max((long long)((nx + ADJ_THREADS - 1) / ADJ_THREADS) * ny,
+                  (long long)((nx + b.x - 1) / b.x) * ((ny + b.y - 1) / b.y));
+}
+
 // One adjoint step (or, with hist_only, the adjoint of the history set-up at
 // t = 0 without the reverse streaming).  state: snapshot of the step's input
-// state (f* set, g* set of pop_bytes each, then the 5 history planes).
+// state (f* set, g* set of pop_bytes each, then the 5 history planes).  At unit
+// rates the compact passes, each a programmatic dependent of the one before.
 template <typename T>
 cudaError_t launch_adjoint_step(const Phys<T>& P, const void* state, long long pop_bytes, const AdjBufs& A,
-                                double* gacc, bool hist_only, cudaStream_t s) {
+                                double* gacc, bool hist_only, bool unit_rates, cudaStream_t s) {
   const T* fin = static_cast<const T*>(state);
   const T* gin = reinterpret_cast<const T*>(static_cast<const unsigned char*>(state) + pop_bytes);
   const T* hist = reinterpret_cast<const T*>(static_cast<const unsigned char*>(state) + 2 * pop_bytes);
-  T* phi = static_cast<T*>(A.phi);
-  T* lext = static_cast<T*>(A.lext);
-  const dim3 grid((P.nx + ADJ_THREADS - 1) / ADJ_THREADS, P.ny);
-  k_adj_phi<T><<<grid, ADJ_THREADS, 0, s>>>(P, fin, phi);
-  k_adj_node<T><<<grid, ADJ_THREADS, 0, s>>>(P, fin, gin, hist, phi, static_cast<const T*>(A.lf),
-                                             static_cast<const T*>(A.lg), static_cast<T*>(A.lh),
-                                             static_cast<T*>(A.lp9), static_cast<T*>(A.lfp),
-                                             static_cast<T*>(A.lgp), A.gpart, hist_only ? 1 : 0);
+  T *phi = static_cast<T*>(A.phi), *lext = static_cast<T*>(A.lext), *lh = static_cast<T*>(A.lh);
+  T *lf = static_cast<T*>(A.lf), *lg = static_cast<T*>(A.lg);
+  T *lp9 = static_cast<T*>(A.lp9), *lfp = static_cast<T*>(A.lfp), *lgp = static_cast<T*>(A.lgp);
+  const dim3 grid((P.nx + ADJ_THREADS - 1) / ADJ_THREADS, P.ny), block(ADJ_THREADS);
   const int ex = P.nx + 2 * P.wall_x, ey = P.ny + 2 * P.wall_y;
-  k_adj_gather<T><<<dim3((ex + ADJ_THREADS - 1) / ADJ_THREADS, ey), ADJ_THREADS, 0, s>>>(
-      P, static_cast<const T*>(A.lp9), lext);
-  if (P.wall_y) k_adj_fold_y<T><<<(ex + ADJ_THREADS - 1) / ADJ_THREADS, ADJ_THREADS, 0, s>>>(P, phi, lext);
-  if (P.wall_x) k_adj_fold_x<T><<<(P.ny + ADJ_THREADS - 1) / ADJ_THREADS, ADJ_THREADS, 0, s>>>(P, phi, lext);
-  if (!hist_only)
-    k_adj_stream<T><<<grid, ADJ_THREADS, 0, s>>>(P, static_cast<const T*>(A.lfp), static_cast<const T*>(A.lgp),
-                                                 lext, static_cast<T*>(A.lf), static_cast<T*>(A.lg));
-  k_adj_reduce<T><<<1, 256, 0, s>>>(A.gpart, (long long)grid.x * grid.y, gacc);
-  return cudaGetLastError();
+  const dim3 egrid((ex + ADJ_THREADS - 1) / ADJ_THREADS, ey);
+  long long parts = (long long)grid.x * grid.y;
+  cudaError_t e = cudaSuccess;
+  if (unit_rates) {
+    const dim3 b = tile_shape<PopPlain<T>>(P.nx, P.ny, false);
+    const dim3 tiles((P.nx + b.x - 1) / b.x, (P.ny + b.y - 1) / b.y);
+    parts = (long long)tiles.x * tiles.y;
+    // (the node pass is a plain launch: the copies and kernels before it on the
+    // stream may write the state or lambda)
+    e = launch_maybe_dependent(false, k_adj_tile<T>, tiles, b, sizeof(T) * (b.x + 2) * (b.y + 2), s, P, fin, gin, hist,
+                               phi, (const T*)lf, (const T*)lg, lh, lp9, lfp, lgp, A.gpart, hist_only ? 1 : 0);
+    if (e == cudaSuccess) e = launch_maybe_dependent(true, k_adj_gather4<T>, egrid, block, 0, s, P, (const T*)lp9, lext);
+  } else {
+    k_adj_phi<T><<<grid, block, 0, s>>>(P, fin, phi);
+    k_adj_node<T><<<grid, block, 0, s>>>(P, fin, gin, hist, phi, lf, lg, lh, lp9, lfp, lgp, A.gpart, hist_only ? 1 : 0);
+    k_adj_gather<T><<<egrid, block, 0, s>>>(P, lp9, lext);
+    e = cudaGetLastError();
+  }
+  if (e == cudaSuccess && P.wall_y)
+    e = launch_maybe_dependent(unit_rates, k_adj_fold_y<T>, dim3((ex + ADJ_THREADS - 1) / ADJ_THREADS), block, 0, s, P,
+                               (const T*)phi, lext);
+  if (e == cudaSuccess && P.wall_x)
+    e = launch_maybe_dependent(unit_rates, k_adj_fold_x<T>, dim3((P.ny + ADJ_THREADS - 1) / ADJ_THREADS), block, 0, s,
+                               P, (const T*)phi, lext);
+  if (e == cudaSuccess && !hist_only) {
+    if (unit_rates) {
+      e = launch_maybe_dependent(true, k_adj_stream14<T>, grid, block, 0, s, P, (const T*)lfp, (const T*)lgp,
+                                 (const T*)lext, lf, lg);
+    } else {
+      k_adj_stream<T><<<grid, block, 0, s>>>(P, lfp, lgp, lext, lf, lg);
+      e = cudaGetLastError();
+    }
+  }
+  if (e == cudaSuccess)
+    e = launch_maybe_dependent(unit_rates, k_adj_reduce<T>, dim3(1), dim3(256), 0, s, (const double*)A.gpart, parts, gacc);
+  return e;
 }
 
 template <typename T>
@@ -499,7 +531,8 @@ cudaError_t launch_adjoint_init(const Phys<T>& P, const AdjBufs& A, double* out,
   template cudaError_t launch_diag<T>(const Phys<T>&, const T*, const T*, double*, int, double*,  \
                                       cudaStream_t);                                             \
   template cudaError_t launch_adjoint_step<T>(const Phys<T>&, const void*, long long, const AdjBufs&, \
-                                              double*, bool, cudaStream_t);                       \
+                                              double*, bool, bool, cudaStream_t);                 \
+  template long long adjoint_blocks<T>(int, int);                                                   \
   template cudaError_t launch_adjoint_seed<T>(const Phys<T>&, const double*, const AdjBufs&,      \
                                               cudaStream_t);                                      \
   template cudaError_t launch_adjoint_init<T>(const Phys<T>&, const AdjBufs&, double*, cudaStream_t); \

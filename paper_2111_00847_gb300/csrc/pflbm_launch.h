@@ -70,7 +70,9 @@ cudaError_t launch_obs(int model, int mode, const Phys<typename C::value_t>& P, 
 // discrete adjoint of the Allen-Cahn step (pflbm_adjoint.cuh), plain storage
 template <typename T>
 cudaError_t launch_adjoint_step(const Phys<T>& P, const void* state, long long pop_bytes, const AdjBufs& A,
-                                double* gacc, bool hist_only, cudaStream_t s);
+                                double* gacc, bool hist_only, bool unit_rates, cudaStream_t s);
+template <typename T>
+long long adjoint_blocks(int nx, int ny);
 template <typename T>
 cudaError_t launch_adjoint_seed(const Phys<T>& P, const double* djdphi, const AdjBufs& A, cudaStream_t s);
 template <typename T>
