@@ -240,7 +240,7 @@ static Phys<T> make_phys(const lbm_handle* h) {
   // its 4th power in T; in FP64 kept above the subnormals (the reciprocal
   // root's hardware seed flushes them), where it regularises nothing
   P.n_delta4 = (P.n_delta * P.n_delta) * (P.n_delta * P.n_delta);
-  if (sizeof(T) == 8) P.n_delta4 = std::max(P.n_delta4, T(1e-290));
+  if constexpr (sizeof(T) == 8) P.n_delta4 = std::max(P.n_delta4, 1e-290);
   P.drho = T(h->drho);
   P.rhoB = T(Q.rhoB);
   P.rho_mean = T(0.5 * (Q.rhoA + Q.rhoB));
@@ -331,17 +331,18 @@ static int ensure_macro(lbm_handle* h) {
   return LBM_OK;
 }
 
-// A kernel whose bounded wait timed out raised *derr; report it once the
-// stream has been synchronised.
+// A kernel whose bounded wait timed out raised *derr: report it (the stream has
+// been synchronised) and clear it.
+static int device_flag_raised(lbm_handle* h) {
+  cudaMemsetAsync(h->derr, 0, sizeof(int), h->stream);
+  return fail(h, LBM_ECUDA, "a step kernel gave up waiting for its staged rows (results since the last check are invalid)");
+}
+// Synchronises the stream.
 static int check_device_flag(lbm_handle* h) {
   int flag = 0;
   CUDA_TRY(h, cudaMemcpyAsync(&flag, h->derr, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
   CUDA_TRY(h, cudaStreamSynchronize(h->stream));
-  if (flag) {
-    cudaMemsetAsync(h->derr, 0, sizeof(int), h->stream);
-    return fail(h, LBM_ECUDA, "a step kernel gave up waiting for its staged rows (results since the last check are invalid)");
-  }
-  return LBM_OK;
+  return flag ? device_flag_raised(h) : LBM_OK;
 }
 
 // Whether the handle's passes run one node per thread (k_tile): plain storage,
@@ -385,12 +386,12 @@ static int run_diag(lbm_handle* h) {
   int rc = run_macro<C>(h);
   if (rc) return rc;
   const Phys<T> P = make_phys<T>(h);
-  CUDA_TRY(h, launch_diag<T>(P, (const T*)h->macro, (const T*)h->phi_prev, h->dpart, h->nparts, h->ddiag, h->stream));
-  double r[DIAG_FIELDS];
+  CUDA_TRY(h, launch_diag<T>(P, (const T*)h->macro, (const T*)h->phi_prev, h->dpart, h->nparts, h->derr, h->ddiag,
+                             h->stream));
+  double r[DIAG_FIELDS + 1];  // the totals and the step kernels' time-out flag
   CUDA_TRY(h, cudaMemcpyAsync(r, h->ddiag, sizeof(r), cudaMemcpyDeviceToHost, h->stream));
   CUDA_TRY(h, cudaStreamSynchronize(h->stream));
-  int rc2 = check_device_flag(h);
-  if (rc2) return rc2;
+  if (r[DIAG_FIELDS] != 0.0) return device_flag_raised(h);
   const double n = r[5];
   h->diag[0] = (double)h->t;
   h->diag[1] = r[0];
@@ -511,8 +512,7 @@ static int export_planes(lbm_handle* h, const T* src, int NP, int k0, int planes
                                  h->stream));
     CUDA_TRY(h, cudaMemcpyAsync(out + k * N, h->dstage, N * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
   }
-  CUDA_TRY(h, cudaStreamSynchronize(h->stream));
-  return check_device_flag(h);
+  return check_device_flag(h);  // synchronises
 }
 
 // host doubles -> all NP planes of an interleaved set (plane 0 minus sub0)
@@ -542,8 +542,7 @@ static int export_pulled(lbm_handle* h, int set, double* out, Region r, double* 
                                       h->stream));
     CUDA_TRY(h, cudaMemcpyAsync(out + k * N, stage, N * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
   }
-  CUDA_TRY(h, cudaStreamSynchronize(h->stream));
-  return check_device_flag(h);
+  return check_device_flag(h);  // synchronises
 }
 
 template <class C>
@@ -764,7 +763,7 @@ static int create_impl(const lbm_params* params, void* stream, const lbm_allocat
   const long long N = (long long)h->nx * h->ny;
   h->nparts = (int)std::min<long long>((N + DIAG_THREADS - 1) / DIAG_THREADS, 152 * 8);
   ok = ok && (h->dpart = (double*)dev_alloc(h, (size_t)h->nparts * DIAG_FIELDS * sizeof(double)));
-  ok = ok && (h->ddiag = (double*)dev_alloc(h, DIAG_FIELDS * sizeof(double)));
+  ok = ok && (h->ddiag = (double*)dev_alloc(h, (DIAG_FIELDS + 1) * sizeof(double)));
   ok = ok && (h->derr = (int*)dev_alloc(h, sizeof(int)));
   if (!ok) {
     std::string msg = "device allocation of " + std::to_string(h->bytes) + " bytes failed";
@@ -1019,8 +1018,7 @@ static int do_fields_noalloc(lbm_handle* h, int which, double* out, double* stag
     CUDA_TRY(h, launch_export<T>(P, src, NP, k, stage, k == 0 ? add0 : 0.0, 0, 0, h->nx, h->ny, h->stream));
     CUDA_TRY(h, cudaMemcpyAsync(out + k * N, stage, N * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
   }
-  CUDA_TRY(h, cudaStreamSynchronize(h->stream));
-  return check_device_flag(h);
+  return check_device_flag(h);  // synchronises
 }
 
 extern "C" int lbm_fields_noalloc(lbm_handle* h, int32_t which, double* out) {
@@ -1046,6 +1044,9 @@ extern "C" int lbm_fields_noalloc(lbm_handle* h, int32_t which, double* out) {
 static long long state_bytes(const lbm_handle* h) {
   return 2 * h->pop_bytes + 5LL * h->plane * (long long)h->esize;
 }
+
+// states up to this size are copied by one kernel
+static constexpr long long COPY_KERNEL_BYTES = 64LL << 20;
 
 static int ensure_adjoint(lbm_handle* h) {
   if (h->have_adj) return LBM_OK;
@@ -1114,8 +1115,46 @@ static int do_adjoint_init(lbm_handle* h, const void* state0, double* out) {
   CUDA_TRY(h, launch_adjoint_init<T>(P, h->adj, h->dstage, h->stream));
   const long long N = (long long)h->nx * h->ny;
   CUDA_TRY(h, cudaMemcpyAsync(out, h->dstage, N * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
-  CUDA_TRY(h, cudaStreamSynchronize(h->stream));
-  return check_device_flag(h);
+  return check_device_flag(h);  // synchronises
+}
+
+// One copy of the three parts of a state (f*, g*, history; a, b, c at offsets 0,
+// na, na + nb of the buffer, in 16-byte words), either way.  Three copy commands
+// take 2 to 3 us each on the stream whatever their size, as long as a whole
+// step of a small grid; above tens of MB one command per part is as fast.
+__global__ void __launch_bounds__(256) k_copy_state(uint4* __restrict__ a, uint4* __restrict__ b, uint4* __restrict__ c,
+                                                    uint4* __restrict__ buf, long long na, long long nb, long long nc,
+                                                    int to_buf) {
+  const long long n = na + nb + nc, step = (long long)gridDim.x * blockDim.x;
+  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += step) {
+    uint4* const p = i < na ? a + i : (i < na + nb ? b + (i - na) : c + (i - na - nb));
+    if (to_buf) buf[i] = *p;
+    else *p = buf[i];
+  }
+}
+
+// Copies the state to or from buf (device memory), on the handle's stream.
+static int copy_state(lbm_handle* h, void* buf, bool to_buf) {
+  void* const part[3] = {h->pops[0][h->cur], h->pops[1][h->cur], h->hist};
+  const long long n[3] = {h->pop_bytes, h->pop_bytes, 5LL * h->plane * (long long)h->esize};
+  unsigned char* p = static_cast<unsigned char*>(buf);
+  if (state_bytes(h) <= COPY_KERNEL_BYTES && (uintptr_t)buf % 16 == 0) {
+    // the kernel touches memory of this device only (parts are 16-byte
+    // multiples: the pitch is a multiple of 32 elements)
+    cudaPointerAttributes at;
+    if (cudaPointerGetAttributes(&at, buf) == cudaSuccess && at.type == cudaMemoryTypeDevice && at.device == h->device) {
+      const long long words = state_bytes(h) / 16;
+      const int blocks = (int)std::min<long long>((words + 255) / 256, 152 * 8);
+      k_copy_state<<<blocks, 256, 0, h->stream>>>((uint4*)part[0], (uint4*)part[1], (uint4*)part[2], (uint4*)buf,
+                                                  n[0] / 16, n[1] / 16, n[2] / 16, to_buf ? 1 : 0);
+      CUDA_TRY(h, cudaGetLastError());
+      return LBM_OK;
+    }
+    cudaGetLastError();
+  }
+  for (int k = 0; k < 3; p += n[k], ++k)
+    CUDA_TRY(h, cudaMemcpyAsync(to_buf ? p : part[k], to_buf ? part[k] : p, n[k], cudaMemcpyDeviceToDevice, h->stream));
+  return LBM_OK;
 }
 
 extern "C" {
@@ -1125,24 +1164,14 @@ int64_t lbm_state_bytes(const lbm_handle* h) { return h ? state_bytes(h) : 0; }
 int lbm_snapshot(lbm_handle* h, void* dst) {
   if (!h) return fail(nullptr, LBM_EINVAL, "handle is NULL");
   if (!dst) return fail(h, LBM_EINVAL, "dst is NULL");
-  unsigned char* d = static_cast<unsigned char*>(dst);
-  CUDA_TRY(h, cudaMemcpyAsync(d, h->pops[0][h->cur], h->pop_bytes, cudaMemcpyDeviceToDevice, h->stream));
-  CUDA_TRY(h, cudaMemcpyAsync(d + h->pop_bytes, h->pops[1][h->cur], h->pop_bytes, cudaMemcpyDeviceToDevice,
-                              h->stream));
-  CUDA_TRY(h, cudaMemcpyAsync(d + 2 * h->pop_bytes, h->hist, 5 * h->plane * h->esize, cudaMemcpyDeviceToDevice,
-                              h->stream));
-  return LBM_OK;
+  return copy_state(h, dst, true);
 }
 
 int lbm_restore(lbm_handle* h, const void* src, int64_t t) {
   if (!h) return fail(nullptr, LBM_EINVAL, "handle is NULL");
   if (!src || t < 0) return fail(h, LBM_EINVAL, "src is NULL or t < 0");
-  const unsigned char* s = static_cast<const unsigned char*>(src);
-  CUDA_TRY(h, cudaMemcpyAsync(h->pops[0][h->cur], s, h->pop_bytes, cudaMemcpyDeviceToDevice, h->stream));
-  CUDA_TRY(h, cudaMemcpyAsync(h->pops[1][h->cur], s + h->pop_bytes, h->pop_bytes, cudaMemcpyDeviceToDevice,
-                              h->stream));
-  CUDA_TRY(h, cudaMemcpyAsync(h->hist, s + 2 * h->pop_bytes, 5 * h->plane * h->esize, cudaMemcpyDeviceToDevice,
-                              h->stream));
+  int rc = copy_state(h, const_cast<void*>(src), false);
+  if (rc) return rc;
   h->t = t;
   return LBM_OK;
 }
@@ -1182,8 +1211,7 @@ int lbm_adjoint_gravity(lbm_handle* h, double* dJ_dG) {
   if (!dJ_dG) return fail(h, LBM_EINVAL, "dJ_dG is NULL");
   if (!h->have_adj) return fail(h, LBM_EINVAL, "lbm_adjoint_seed has not been called");
   CUDA_TRY(h, cudaMemcpyAsync(dJ_dG, h->gacc, 2 * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
-  CUDA_TRY(h, cudaStreamSynchronize(h->stream));
-  return check_device_flag(h);
+  return check_device_flag(h);  // synchronises
 }
 
 }  // extern "C"

@@ -2864,6 +2864,8 @@ template <typename T>
 __global__ void __launch_bounds__(DIAG_THREADS) k_diag_partial(const Phys<T> P, const T* __restrict__ mac,
                                                                const T* __restrict__ phi_prev,
                                                                double* __restrict__ partial) {
+  asm volatile("griddepcontrol.launch_dependents;");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   double v[DIAG_FIELDS] = {0, 0, 0, 0, 0, 0};
   const long long N = (long long)P.nx * P.diag_y1;
   const long long pl = P.pitch;  // macro plane k of a node sits k * pitch after plane 0
@@ -2908,9 +2910,13 @@ __global__ void __launch_bounds__(DIAG_THREADS) k_diag_partial(const Phys<T> P, 
   block_reduce6(v, partial + (long long)blockIdx.x * DIAG_FIELDS);
 }
 
+// The totals, and after them the time-out flag of the step kernels, so that one
+// copy brings both to the host.
 template <typename T>
-__global__ void __launch_bounds__(DIAG_THREADS) k_diag_final(const double* __restrict__ partial,
-                                                             int nparts, double* __restrict__ out) {
+__global__ void __launch_bounds__(DIAG_THREADS) k_diag_final(const double* __restrict__ partial, int nparts,
+                                                             const int* __restrict__ err, double* __restrict__ out) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (threadIdx.x == 0) out[DIAG_FIELDS] = double(*err);
   double v[DIAG_FIELDS] = {0, 0, 0, 0, 0, 0};
   for (int b = threadIdx.x; b < nparts; b += blockDim.x) {
 #pragma unroll

@@ -288,12 +288,16 @@ cudaError_t launch_import(const Phys<T>& P, const double* in, T* out, int NP, in
   return cudaGetLastError();
 }
 
+// (each a programmatic dependent of the kernel before it)
 template <typename T>
-cudaError_t launch_diag(const Phys<T>& P, const T* macro, const T* phi_prev, double* partial,
-                        int nparts, double* out, cudaStream_t s) {
-  k_diag_partial<T><<<nparts, DIAG_THREADS, 0, s>>>(P, macro, phi_prev, partial);
-  k_diag_final<T><<<1, DIAG_THREADS, 0, s>>>(partial, nparts, out);
-  return cudaGetLastError();
+cudaError_t launch_diag(const Phys<T>& P, const T* macro, const T* phi_prev, double* partial, int nparts,
+                        const int* err, double* out, cudaStream_t s) {
+  cudaError_t e = launch_maybe_dependent(true, k_diag_partial<T>, dim3(nparts), dim3(DIAG_THREADS), 0, s, P, macro,
+                                         phi_prev, partial);
+  if (e == cudaSuccess)
+    e = launch_maybe_dependent(true, k_diag_final<T>, dim3(1), dim3(DIAG_THREADS), 0, s, (const double*)partial, nparts,
+                               err, out);
+  return e;
 }
 
 template <typename T>
@@ -528,8 +532,8 @@ cudaError_t launch_adjoint_init(const Phys<T>& P, const AdjBufs& A, double* out,
                                         int, int, int, cudaStream_t);                              \
   template cudaError_t launch_import<T>(const Phys<T>&, const double*, T*, int, int, double,      \
                                         cudaStream_t);                                             \
-  template cudaError_t launch_diag<T>(const Phys<T>&, const T*, const T*, double*, int, double*,  \
-                                      cudaStream_t);                                             \
+  template cudaError_t launch_diag<T>(const Phys<T>&, const T*, const T*, double*, int, const int*, \
+                                      double*, cudaStream_t);                                      \
   template cudaError_t launch_adjoint_step<T>(const Phys<T>&, const void*, long long, const AdjBufs&, \
                                               double*, bool, bool, cudaStream_t);                 \
   template long long adjoint_blocks<T>(int, int);                                                   \

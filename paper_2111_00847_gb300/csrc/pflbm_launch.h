@@ -54,8 +54,8 @@ template <typename T>
 cudaError_t launch_import(const Phys<T>& P, const double* in, T* out, int NP, int k, double sub,
                           cudaStream_t s);
 template <typename T>
-cudaError_t launch_diag(const Phys<T>& P, const T* macro, const T* phi_prev, double* partial,
-                        int nparts, double* out, cudaStream_t s);
+cudaError_t launch_diag(const Phys<T>& P, const T* macro, const T* phi_prev, double* partial, int nparts,
+                        const int* err, double* out, cudaStream_t s);
 // solid obstacles (pflbm_obstacle.cuh): the reflecting links of every node
 // from a dense byte mask, and one step (or MACRO / HIST / INIT pass) through
 // the obstacle passes; phis, mus: one-plane work planes of the arithmetic
