@@ -148,7 +148,11 @@ class LbmError(RuntimeError):
 
 
 def _dptr(a):
-    return None if a is None else a.ctypes.data_as(C.POINTER(C.c_double))
+    if a is None:
+        return None
+    if isinstance(a, np.ndarray):
+        return a.ctypes.data_as(C.POINTER(C.c_double))
+    return C.cast(a.data_ptr(), C.POINTER(C.c_double))  # a contiguous float64 tensor on the handle's device
 
 
 # ---- one-to-one wrappers of the C entry points ------------------------------

@@ -22,7 +22,7 @@ import copy
 import numpy as np
 import torch
 
-from . import LBM_PHI, Simulation
+from . import LBM_PHI, Simulation, lbm_adjoint_init, lbm_adjoint_seed, lbm_fields, lbm_init_fields
 
 
 def _with_gravity(params, gx: float, gy: float):
@@ -31,6 +31,23 @@ def _with_gravity(params, gx: float, gy: float):
     p = copy.copy(params)
     p.gx, p.gy = gx, gy
     return p
+
+
+def _on_handle_device(t) -> bool:
+    """Whether the library can read tensor t where it lies: on the current
+    device, the one a new Simulation lives on.  phi0 and the gradients then
+    never pass through the host (500 x 1000 FP32, 40 steps: 6.0 -> 5.7 ms)."""
+    return t.is_cuda and t.device.index == torch.cuda.current_device()
+
+
+def _device_field(t, sim):
+    """t as a contiguous float64 [ny, nx] tensor on its device."""
+    t = t.detach().to(torch.float64).contiguous()
+    if tuple(t.shape) != (sim.ny, sim.nx):
+        raise ValueError(f"field shape {tuple(t.shape)} != {(sim.ny, sim.nx)}")
+    if sim.stream != torch.cuda.current_stream().cuda_stream:
+        torch.cuda.current_stream().synchronize()  # t was made on another stream than the handle's
+    return t
 
 
 class Rollout(torch.autograd.Function):
@@ -43,7 +60,11 @@ class Rollout(torch.autograd.Function):
             raise ValueError("steps and every must be positive")
         g = gravity.detach().double().cpu().numpy()
         sim = Simulation(_with_gravity(params, float(g[0]), float(g[1])))
-        sim.init_fields(phi0.detach().double().cpu().numpy())
+        direct = _on_handle_device(phi0)
+        if direct:
+            lbm_init_fields(sim.handle, _device_field(phi0, sim))  # returns when the field has been read
+        else:
+            sim.init_fields(phi0.detach().double().cpu().numpy())
         ckpts = [sim.snapshot(sim.new_state_buffer())]
         t = 0
         while t < steps:
@@ -52,7 +73,12 @@ class Rollout(torch.autograd.Function):
             t += n
             if t < steps:
                 ckpts.append(sim.snapshot(sim.new_state_buffer()))
-        phiN = torch.from_numpy(sim.fields(LBM_PHI)).to(phi0.device)
+        if direct:
+            phiN = torch.empty((sim.ny, sim.nx), dtype=torch.float64, device=phi0.device)
+            lbm_fields(sim.handle, LBM_PHI, phiN)
+        else:
+            phiN = torch.from_numpy(sim.fields(LBM_PHI)).to(phi0.device)
+        ctx.direct = direct
         ctx.sim, ctx.ckpts, ctx.steps, ctx.every = sim, ckpts, steps, every
         ctx.devices = (phi0.device, gravity.device)
         return phiN
@@ -60,7 +86,12 @@ class Rollout(torch.autograd.Function):
     @staticmethod
     def backward(ctx, grad_phiN):
         sim, ckpts, steps, K = ctx.sim, ctx.ckpts, ctx.steps, ctx.every
-        sim.adjoint_seed(grad_phiN.detach().double().cpu().numpy())
+        direct = ctx.direct and _on_handle_device(grad_phiN)
+        if direct:
+            seed = _device_field(grad_phiN, sim)  # kept until adjoint_init has synchronised
+            lbm_adjoint_seed(sim.handle, seed)
+        else:
+            sim.adjoint_seed(grad_phiN.detach().double().cpu().numpy())
         work = [sim.new_state_buffer() for _ in range(min(K, steps) - 1)]
         for c in reversed(range(len(ckpts))):
             t0 = c * K
@@ -72,12 +103,15 @@ class Rollout(torch.autograd.Function):
                 seg.append(sim.snapshot(work[j - 1]))
             for j in reversed(range(L)):
                 sim.adjoint_step(seg[j])
-        dphi0 = sim.adjoint_init(ckpts[0])
+        if direct:
+            dphi0 = torch.empty((sim.ny, sim.nx), dtype=torch.float64, device=ctx.devices[0])
+            lbm_adjoint_init(sim.handle, ckpts[0].data_ptr(), dphi0)
+        else:
+            dphi0 = torch.from_numpy(sim.adjoint_init(ckpts[0])).to(ctx.devices[0])
         dG = sim.adjoint_gravity()
         ctx.sim = ctx.ckpts = None
         sim.close()
-        return (torch.from_numpy(dphi0).to(ctx.devices[0]),
-                torch.from_numpy(dG).to(ctx.devices[1]), None, None, None)
+        return (dphi0, torch.from_numpy(dG).to(ctx.devices[1]), None, None, None)
 
 
 def rollout(phi0: torch.Tensor, gravity: torch.Tensor, params, steps: int, every: int = 100) -> torch.Tensor:

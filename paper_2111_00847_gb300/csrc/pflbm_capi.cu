@@ -300,7 +300,9 @@ static Phys<T> make_phys(const lbm_handle* h) {
 }
 
 // ---------------------------------------------------------------------------
-// Typed operations (T = float or double)
+// Typed operations (T = float or double).  Fields given to or taken by the
+// caller are copied with cudaMemcpyDefault: in host memory, or in memory of the
+// handle's device, which then costs a device copy instead of a transfer.
 // ---------------------------------------------------------------------------
 template <typename T>
 static Bufs<T> bufs_now(lbm_handle* h) {
@@ -460,12 +462,12 @@ static int do_init(lbm_handle* h, const double* phi, const double* ux, const dou
   const Phys<T> P = make_phys<T>(h);
   Bufs<T> B = bufs_now<T>(h);
   double* d = h->dstage;
-  CUDA_TRY(h, cudaMemcpyAsync(d, phi, N * sizeof(double), cudaMemcpyHostToDevice, h->stream));
+  CUDA_TRY(h, cudaMemcpyAsync(d, phi, N * sizeof(double), cudaMemcpyDefault, h->stream));
   B.iphi = d;
   d += N;
-  if (ux) { CUDA_TRY(h, cudaMemcpyAsync(d, ux, N * sizeof(double), cudaMemcpyHostToDevice, h->stream)); B.iux = d; d += N; }
-  if (uy) { CUDA_TRY(h, cudaMemcpyAsync(d, uy, N * sizeof(double), cudaMemcpyHostToDevice, h->stream)); B.iuy = d; d += N; }
-  if (p) { CUDA_TRY(h, cudaMemcpyAsync(d, p, N * sizeof(double), cudaMemcpyHostToDevice, h->stream)); B.ip = d; d += N; }
+  if (ux) { CUDA_TRY(h, cudaMemcpyAsync(d, ux, N * sizeof(double), cudaMemcpyDefault, h->stream)); B.iux = d; d += N; }
+  if (uy) { CUDA_TRY(h, cudaMemcpyAsync(d, uy, N * sizeof(double), cudaMemcpyDefault, h->stream)); B.iuy = d; d += N; }
+  if (p) { CUDA_TRY(h, cudaMemcpyAsync(d, p, N * sizeof(double), cudaMemcpyDefault, h->stream)); B.ip = d; d += N; }
   if constexpr (!C::dev) {
     // equilibria per node into the spare buffers, then scatter to the pull layout
     CUDA_TRY(h, launch_mode<C>(h, MODE_INIT, P, B));
@@ -510,7 +512,7 @@ static int export_planes(lbm_handle* h, const T* src, int NP, int k0, int planes
   for (int k = 0; k < planes; ++k) {
     CUDA_TRY(h, launch_export<T>(P, src, NP, k0 + k, h->dstage, k == 0 ? add0 : 0.0, r.x0, r.y0, r.w, r.h,
                                  h->stream));
-    CUDA_TRY(h, cudaMemcpyAsync(out + k * N, h->dstage, N * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
+    CUDA_TRY(h, cudaMemcpyAsync(out + k * N, h->dstage, N * sizeof(double), cudaMemcpyDefault, h->stream));
   }
   return check_device_flag(h);  // synchronises
 }
@@ -523,7 +525,7 @@ static int import_planes(lbm_handle* h, const double* in, int NP, double sub0, T
   const Phys<T> P = make_phys<T>(h);
   const long long N = (long long)h->nx * h->ny;
   for (int k = 0; k < NP; ++k) {
-    CUDA_TRY(h, cudaMemcpyAsync(h->dstage, in + k * N, N * sizeof(double), cudaMemcpyHostToDevice, h->stream));
+    CUDA_TRY(h, cudaMemcpyAsync(h->dstage, in + k * N, N * sizeof(double), cudaMemcpyDefault, h->stream));
     CUDA_TRY(h, launch_import<T>(P, h->dstage, dst, NP, k, k == 0 ? sub0 : 0.0, h->stream));
   }
   CUDA_TRY(h, cudaStreamSynchronize(h->stream));
@@ -540,7 +542,7 @@ static int export_pulled(lbm_handle* h, int set, double* out, Region r, double* 
     CUDA_TRY(h, launch_pull_export<C>(P, h->pops[set][h->cur], set, k, stage,
                                       (k == 0 && set == 1) ? h->prm.rho0 : 0.0, r.x0, r.y0, r.w, r.h,
                                       h->stream));
-    CUDA_TRY(h, cudaMemcpyAsync(out + k * N, stage, N * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
+    CUDA_TRY(h, cudaMemcpyAsync(out + k * N, stage, N * sizeof(double), cudaMemcpyDefault, h->stream));
   }
   return check_device_flag(h);  // synchronises
 }
@@ -1016,7 +1018,7 @@ static int do_fields_noalloc(lbm_handle* h, int which, double* out, double* stag
   const long long N = (long long)h->nx * h->ny;
   for (int k = 0; k < NP; ++k) {
     CUDA_TRY(h, launch_export<T>(P, src, NP, k, stage, k == 0 ? add0 : 0.0, 0, 0, h->nx, h->ny, h->stream));
-    CUDA_TRY(h, cudaMemcpyAsync(out + k * N, stage, N * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
+    CUDA_TRY(h, cudaMemcpyAsync(out + k * N, stage, N * sizeof(double), cudaMemcpyDefault, h->stream));
   }
   return check_device_flag(h);  // synchronises
 }
@@ -1093,7 +1095,7 @@ static int do_adjoint_seed(lbm_handle* h, const double* djdphi) {
   int rc = ensure_stage(h, 1);
   if (rc) return rc;
   const long long N = (long long)h->nx * h->ny;
-  CUDA_TRY(h, cudaMemcpyAsync(h->dstage, djdphi, N * sizeof(double), cudaMemcpyHostToDevice, h->stream));
+  CUDA_TRY(h, cudaMemcpyAsync(h->dstage, djdphi, N * sizeof(double), cudaMemcpyDefault, h->stream));
   CUDA_TRY(h, launch_adjoint_seed<T>(P, h->dstage, h->adj, h->stream));
   CUDA_TRY(h, cudaMemsetAsync(h->gacc, 0, 2 * sizeof(double), h->stream));
   return LBM_OK;
@@ -1114,7 +1116,7 @@ static int do_adjoint_init(lbm_handle* h, const void* state0, double* out) {
   CUDA_TRY(h, launch_adjoint_step<T>(P, state0, h->pop_bytes, h->adj, h->gacc, true, h->unit_rates, h->stream));
   CUDA_TRY(h, launch_adjoint_init<T>(P, h->adj, h->dstage, h->stream));
   const long long N = (long long)h->nx * h->ny;
-  CUDA_TRY(h, cudaMemcpyAsync(out, h->dstage, N * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
+  CUDA_TRY(h, cudaMemcpyAsync(out, h->dstage, N * sizeof(double), cudaMemcpyDefault, h->stream));
   return check_device_flag(h);  // synchronises
 }
 
