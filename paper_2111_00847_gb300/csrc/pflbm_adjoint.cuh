@@ -812,6 +812,63 @@ __device__ __forceinline__ void node_adjoint_unit(const Phys<T>& P, const Row3<T
   o4[3] = lgy;
 }
 
+// Wetting ghosts of a phi tile (as in k_tile; after a barrier, ends with one where
+// there are any): the column beyond an x wall on every row the tile and its halo hold,
+// then the row beyond a y wall over the widened columns.  cl, cr, rb, rt: their
+// places relative to the tile (block-uniform; a Cahn-Hilliard tile that ends one
+// node short of a wall holds the ghosts too, for mu_phi of the node between).
+template <int R, typename T>
+__device__ __forceinline__ void tile_ghosts(const Phys<T>& P, T* sp, int pw, int x0, int y0, int w, int hgt, int tid,
+                                            int nth) {
+  const bool wx = P.wall_x != 0, wy = P.wall_y != 0;
+  const int cl = -1 - x0, cr = P.nx - x0, rb = -1 - y0, rt = P.ny - y0;
+  const bool has_l = wx && cl >= -R, has_r = wx && cr < w + R;
+  const bool has_b = wy && rb >= -R, has_t = wy && rt < hgt + R;
+  if (has_l || has_r) {
+    for (int r = tid; r < hgt + 2 * R; r += nth) {
+      T* const q = sp + r * pw + R;
+      if (has_l) q[cl] = wall_ghost(P, SIDE_LEFT, q[cl + 1], q[cl + 2]);
+      if (has_r) q[cr] = wall_ghost(P, SIDE_RIGHT, q[cr - 1], q[cr - 2]);
+    }
+    __syncthreads();
+  }
+  if (has_b || has_t) {
+    for (int c = tid; c < w + 2 * R; c += nth) {
+      T* const q = sp + R * pw + c;
+      if (has_b) q[rb * pw] = wall_ghost(P, SIDE_BOTTOM, q[(rb + 1) * pw], q[(rb + 2) * pw]);
+      if (has_t) q[rt * pw] = wall_ghost(P, SIDE_TOP, q[(rt - 1) * pw], q[(rt - 2) * pw]);
+    }
+    __syncthreads();
+  }
+}
+
+// phi of a tile's halo ring (in the domain, or wrapped), as k_tile forms it on
+// tiles at the grid's edge (written out there: as a call it cost the
+// Cahn-Hilliard step 100 bytes of spills, 4096^2 592 -> 670 us).
+template <class C, int MODE, int R, typename T = typename C::value_t>
+__device__ __forceinline__ void tile_ring(const Phys<T>& P, const Bufs<T>& B, T* sp, int pw, int x0, int y0, int w,
+                                          int hgt, int tid, int nth) {
+  const int nx = P.nx, ny = P.ny;
+  const bool wx = P.wall_x != 0, wy = P.wall_y != 0;
+  const int row_cells = R * (w + 2 * R), ring = 2 * row_cells + 2 * R * hgt;
+  for (int k = tid; k < ring; k += nth) {
+    int cx, cy;
+    if (k < 2 * row_cells) {
+      const int r = k / (w + 2 * R);
+      cx = k - r * (w + 2 * R) - R;
+      cy = r < R ? r - R : hgt + (r - R);
+    } else {
+      const int q = k - 2 * row_cells, r = q / (2 * R), c = q - r * 2 * R;
+      cy = r;
+      cx = c < R ? c - R : w + (c - R);
+    }
+    int xx = x0 + cx, yy = y0 + cy;
+    if ((wx && (xx < 0 || xx >= nx)) || (wy && (yy < 0 || yy >= ny))) continue;  // ghosts follow
+    xx = xx < 0 ? xx + nx : (xx >= nx ? xx - nx : xx);
+    yy = yy < 0 ? yy + ny : (yy >= ny ? yy - ny : yy);
+    sp[(cy + R) * pw + cx + R] = phi_at<C, MODE>(P, B, xx, yy);
+  }
+}
 template <typename T>
 __global__ void __launch_bounds__(TILE_THREADS, 2)
     k_adj_tile(const Phys<T> P, const T* __restrict__ fin, const T* __restrict__ gin, const T* __restrict__ hist,
@@ -828,30 +885,80 @@ __global__ void __launch_bounds__(TILE_THREADS, 2)
   const int x = x0 + tx, y = y0 + ty;
   asm volatile("griddepcontrol.launch_dependents;");
   asm volatile("griddepcontrol.wait;" ::: "memory");
+  const bool wx = P.wall_x != 0;
+  // as in k_tile: what an interior tile reads is addressed from block-uniform
+  // bases with one 32-bit offset per node and layout
+  const bool inner = w == bw && hgt == bh && y0 > 1 && y0 + bh + 1 < P.ny && (!wx || (x0 > 1 && x0 + bw + 1 < P.nx));
+  const uint32_t o9 = TileAddr<T>::node(tx, ty, P.pitch);
   T f[9], g[9], lfs[9], lgs[9], lhn[5], h3 = T(0), h4 = T(0);
-  if (active) {
-    pull9<PopPlain<T>>(fin, P, 0, x, y, f);
-    pull9<PopPlain<T>>(gin, P, 1, x, y, g);
-    const long long i9 = ix(P, 9, 0, x, y), i5 = ix(P, 5, 0, x, y), pc = P.pitch;
+  if (inner) {
+    const TileAddr<T> F(fin, P, x0, y0), G(gin, P, x0, y0), A(lf, P, x0, y0), C(lg, P, x0, y0);
+    const int shares = 2 + (2 * (bh + 2) + 31) / 32, warps = (nth + 31) >> 5;
+    auto place = [&](int k, int& cx, int& cy) {
+      cx = tid & 31;
+      if (k < 2) {
+        cy = k == 0 ? -1 : bh;
+        return cx < bw;
+      }
+      const int q = (k - 2) * 32 + cx;
+      cy = q / 2 - 1;
+      cx = (q & 1) ? bw : -1;
+      return cy < bh + 1;
+    };
+    T v[9];
+    int k = tid >> 5, cx, cy;
+    const bool on = k < shares && place(k, cx, cy);
+    if (on) F.pull(TileAddr<T>::node(cx, cy, P.pitch), v);
+    F.pull(o9, f);
+    G.pull(o9, g);
+    const uint32_t o5 = (uint32_t)((ty * 5 * P.pitch + tx) * (int)sizeof(T));
+    const long long pc = (long long)P.pitch * (long long)sizeof(T);
+    const unsigned char* const lb = reinterpret_cast<const unsigned char*>(lh + ix(P, 5, 0, x0, y0));
+    const unsigned char* const hb = reinterpret_cast<const unsigned char*>(hist + ix(P, 5, 0, x0, y0));
 #pragma unroll
     for (int i = 0; i < 9; ++i) {
-      lfs[i] = hist_only ? T(0) : lf[i9 + i * pc];
-      lgs[i] = hist_only ? T(0) : lg[i9 + i * pc];
+      lfs[i] = hist_only ? T(0) : *reinterpret_cast<const T*>(A.base + i * pc + o9);
+      lgs[i] = hist_only ? T(0) : *reinterpret_cast<const T*>(C.base + i * pc + o9);
     }
 #pragma unroll
-    for (int k = 0; k < 5; ++k) lhn[k] = lh[i5 + k * pc];
-    if (!hist_only) h3 = hist[i5 + 3 * pc], h4 = hist[i5 + 4 * pc];
+    for (int i = 0; i < 5; ++i) lhn[i] = *reinterpret_cast<const T*>(lb + i * pc + o5);
+    if (!hist_only) {
+      h3 = *reinterpret_cast<const T*>(hb + 3 * pc + o5);
+      h4 = *reinterpret_cast<const T*>(hb + 4 * pc + o5);
+    }
+    if (on) sp[(cy + 1) * pw + cx + 1] = sum9(v);
+    for (k += warps; k < shares; k += warps) {
+      if (!place(k, cx, cy)) continue;
+      F.pull(TileAddr<T>::node(cx, cy, P.pitch), v);
+      sp[(cy + 1) * pw + cx + 1] = sum9(v);
+    }
+  } else {
+    if (active) {
+      pull9<PopPlain<T>>(fin, P, 0, x, y, f);
+      pull9<PopPlain<T>>(gin, P, 1, x, y, g);
+      const long long i9 = ix(P, 9, 0, x, y), i5 = ix(P, 5, 0, x, y), pc = P.pitch;
+#pragma unroll
+      for (int i = 0; i < 9; ++i) {
+        lfs[i] = hist_only ? T(0) : lf[i9 + i * pc];
+        lgs[i] = hist_only ? T(0) : lg[i9 + i * pc];
+      }
+#pragma unroll
+      for (int k = 0; k < 5; ++k) lhn[k] = lh[i5 + k * pc];
+      if (!hist_only) h3 = hist[i5 + 3 * pc], h4 = hist[i5 + 4 * pc];
+    }
+    Bufs<T> B;
+    B.fin = fin;
+    tile_ring<PopPlain<T>, MODE_STEP, 1>(P, B, sp, pw, x0, y0, w, hgt, tid, nth);
   }
-  Bufs<T> B;
-  B.fin = fin;
-  tile_ring<PopPlain<T>, MODE_STEP, 1>(P, B, sp, pw, x0, y0, w, hgt, tid, nth);
   if (active) {
     const T ph = sum9(f);
     sp[(ty + 1) * pw + tx + 1] = ph;
-    phi[ix(P, 1, 0, x, y)] = ph;  // for the folds of the wetting ghosts
+    // for the folds of the wetting ghosts, which read the two rows and columns
+    // next to a wall
+    if (!inner) phi[ix(P, 1, 0, x, y)] = ph;
   }
   __syncthreads();
-  tile_ghosts<1>(P, sp, pw, x0, y0, w, hgt, tid, nth);
+  if (!inner) tile_ghosts<1>(P, sp, pw, x0, y0, w, hgt, tid, nth);
   T gxs = T(0), gys = T(0);
   if (active) {
     const T* const q = sp + (ty + 1) * pw + tx + 1;

@@ -348,10 +348,10 @@ static int check_device_flag(lbm_handle* h) {
 }
 
 // Whether the handle's passes run one node per thread (k_tile): plain storage,
-// no obstacles.  LBM_FLAG_NO_TMA asks for the register-pipelined kernel.
+// no obstacles, rows it can address.  LBM_FLAG_NO_TMA asks for the register-pipelined kernel.
 template <class C>
 static bool use_tile(const lbm_handle* h) {
-  return !C::dev && h->use_tma && !h->dobs;
+  return !C::dev && h->use_tma && !h->dobs && h->pitch <= TILE_MAX_PITCH;
 }
 
 // One pass of the fused kernel in a mode, or, with solid obstacles, the

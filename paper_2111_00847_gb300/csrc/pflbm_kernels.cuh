@@ -1390,7 +1390,14 @@ __global__ void __launch_bounds__(BX) k_march(const Phys<typename C::value_t> P,
 // and flatter than 4 rows pull more of the ring than they save (4096^2: 64 x 4
 // 543 us, 128 x 1 617).  Kept to 32 columns, a warp is one row.
 // ---------------------------------------------------------------------------
-// Threads and resident blocks per SM it is compiled for.
+// Threads and resident blocks per SM it is compiled for, and the longest rows
+// it takes: a tile's offsets stay below 2^31 bytes (at most (8 + 6) 9 rows of
+// 2^20 FP64 elements; taller tiles are of grids narrower than 32 columns).
+// Longer rows go to k_march.  The test sits on the host, and the tile's slow
+// path below is written out rather than called, because the Cahn-Hilliard
+// kernel at 64 registers answers both with spills or a worse schedule (4096^2:
+// 593 us a step; 634 with the test inside, 680 with the ghosts as a function).
+constexpr int TILE_MAX_PITCH = 1 << 20;
 constexpr int TILE_THREADS = 256;
 template <typename T, int MODEL>
 struct TileCfg {
@@ -1452,62 +1459,6 @@ struct TileSink {
     for (int i = 0; i < 9; ++i) *reinterpret_cast<T*>(s + i * pc + o9) = v[i];
   }
 };
-
-// phi of a tile's halo ring (in the domain, or wrapped): R rows below and above
-// over the widened columns, then R columns on either side.
-template <class C, int MODE, int R, typename T = typename C::value_t>
-__device__ __forceinline__ void tile_ring(const Phys<T>& P, const Bufs<T>& B, T* sp, int pw, int x0, int y0, int w,
-                                          int hgt, int tid, int nth) {
-  const int nx = P.nx, ny = P.ny;
-  const bool wx = P.wall_x != 0, wy = P.wall_y != 0;
-  const int row_cells = R * (w + 2 * R), ring = 2 * row_cells + 2 * R * hgt;
-  for (int k = tid; k < ring; k += nth) {
-    int cx, cy;
-    if (k < 2 * row_cells) {
-      const int r = k / (w + 2 * R);
-      cx = k - r * (w + 2 * R) - R;
-      cy = r < R ? r - R : hgt + (r - R);
-    } else {
-      const int q = k - 2 * row_cells, r = q / (2 * R), c = q - r * 2 * R;
-      cy = r;
-      cx = c < R ? c - R : w + (c - R);
-    }
-    int xx = x0 + cx, yy = y0 + cy;
-    if ((wx && (xx < 0 || xx >= nx)) || (wy && (yy < 0 || yy >= ny))) continue;  // ghosts follow
-    xx = xx < 0 ? xx + nx : (xx >= nx ? xx - nx : xx);
-    yy = yy < 0 ? yy + ny : (yy >= ny ? yy - ny : yy);
-    sp[(cy + R) * pw + cx + R] = phi_at<C, MODE>(P, B, xx, yy);
-  }
-}
-// Wetting ghosts of a phi tile (after a barrier; ends with one where there are
-// any): the column beyond an x wall on every row the tile and its halo hold,
-// then the row beyond a y wall over the widened columns.  cl, cr, rb, rt: their
-// places relative to the tile (block-uniform; a Cahn-Hilliard tile that ends one
-// node short of a wall holds the ghosts too, for mu_phi of the node between).
-template <int R, typename T>
-__device__ __forceinline__ void tile_ghosts(const Phys<T>& P, T* sp, int pw, int x0, int y0, int w, int hgt, int tid,
-                                            int nth) {
-  const bool wx = P.wall_x != 0, wy = P.wall_y != 0;
-  const int cl = -1 - x0, cr = P.nx - x0, rb = -1 - y0, rt = P.ny - y0;
-  const bool has_l = wx && cl >= -R, has_r = wx && cr < w + R;
-  const bool has_b = wy && rb >= -R, has_t = wy && rt < hgt + R;
-  if (has_l || has_r) {
-    for (int r = tid; r < hgt + 2 * R; r += nth) {
-      T* const q = sp + r * pw + R;
-      if (has_l) q[cl] = wall_ghost(P, SIDE_LEFT, q[cl + 1], q[cl + 2]);
-      if (has_r) q[cr] = wall_ghost(P, SIDE_RIGHT, q[cr - 1], q[cr - 2]);
-    }
-    __syncthreads();
-  }
-  if (has_b || has_t) {
-    for (int c = tid; c < w + 2 * R; c += nth) {
-      T* const q = sp + R * pw + c;
-      if (has_b) q[rb * pw] = wall_ghost(P, SIDE_BOTTOM, q[(rb + 1) * pw], q[(rb + 2) * pw]);
-      if (has_t) q[rt * pw] = wall_ghost(P, SIDE_TOP, q[(rt - 1) * pw], q[(rt - 2) * pw]);
-    }
-    __syncthreads();
-  }
-}
 
 // The update of a tile that reaches a solid obstacle (Allen-Cahn STEP; a solid
 // node within 3 nodes of the tile): phi of the fluid nodes up to two nodes out
@@ -1707,10 +1658,52 @@ __global__ void __launch_bounds__(TILE_THREADS, (TileCfg<typename C::value_t, MO
         }
       }
     }
-    tile_ring<C, MODE, R>(P, B, sp, pw, x0, y0, w, hgt, tid, nth);
+    // the halo ring (in the domain, or wrapped): R rows below and above over the
+    // widened columns, then R columns on either side
+    const int row_cells = R * (w + 2 * R), ring = 2 * row_cells + 2 * R * hgt;
+    for (int k = tid; k < ring; k += nth) {
+      int cx, cy;
+      if (k < 2 * row_cells) {
+        const int r = k / (w + 2 * R);
+        cx = k - r * (w + 2 * R) - R;
+        cy = r < R ? r - R : hgt + (r - R);
+      } else {
+        const int q = k - 2 * row_cells, r = q / (2 * R), c = q - r * 2 * R;
+        cy = r;
+        cx = c < R ? c - R : w + (c - R);
+      }
+      int xx = x0 + cx, yy = y0 + cy;
+      if ((wx && (xx < 0 || xx >= nx)) || (wy && (yy < 0 || yy >= ny))) continue;  // ghosts follow
+      xx = xx < 0 ? xx + nx : (xx >= nx ? xx - nx : xx);
+      yy = yy < 0 ? yy + ny : (yy >= ny ? yy - ny : yy);
+      sp[(cy + R) * pw + cx + R] = phi_at<C, MODE>(P, B, xx, yy);
+    }
     if (active) sp[(ty + R) * pw + tx + R] = MODE == MODE_INIT ? T(B.iphi[(long long)y * nx + x]) : sum9(f);
     __syncthreads();
-    tile_ghosts<R>(P, sp, pw, x0, y0, w, hgt, tid, nth);
+    // wetting ghosts: the column beyond an x wall on every row the tile and its
+    // halo hold, then the row beyond a y wall over the widened columns.  cl, cr,
+    // rb, rt: their places relative to the tile (block-uniform; a Cahn-Hilliard
+    // tile that ends one node short of a wall holds the ghosts too, for mu_phi
+    // of the node between)
+    const int cl = -1 - x0, cr = nx - x0, rb = -1 - y0, rt = ny - y0;
+    const bool has_l = wx && cl >= -R, has_r = wx && cr < w + R;
+    const bool has_b = wy && rb >= -R, has_t = wy && rt < hgt + R;
+    if (has_l || has_r) {
+      for (int r = tid; r < hgt + 2 * R; r += nth) {
+        T* const q = sp + r * pw + R;
+        if (has_l) q[cl] = wall_ghost(P, SIDE_LEFT, q[cl + 1], q[cl + 2]);
+        if (has_r) q[cr] = wall_ghost(P, SIDE_RIGHT, q[cr - 1], q[cr - 2]);
+      }
+      __syncthreads();
+    }
+    if (has_b || has_t) {
+      for (int c = tid; c < w + 2 * R; c += nth) {
+        T* const q = sp + R * pw + c;
+        if (has_b) q[rb * pw] = wall_ghost(P, SIDE_BOTTOM, q[(rb + 1) * pw], q[(rb + 2) * pw]);
+        if (has_t) q[rt * pw] = wall_ghost(P, SIDE_TOP, q[(rt - 1) * pw], q[(rt - 2) * pw]);
+      }
+      __syncthreads();
+    }
   }
   if (MODEL == MODEL_CH) {
     // mu_phi on the tile and one node around it; beyond walls the mirror value

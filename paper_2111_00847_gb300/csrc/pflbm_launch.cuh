@@ -415,8 +415,7 @@ cudaError_t launch_obs(int model, int mode, const Phys<typename C::value_t>& P, 
   if (!P.obs || !phis || (model == MODEL_CH && !mus)) return cudaErrorInvalidValue;
   if (use_tma && model == MODEL_AC && mode == MODE_STEP && P.nx >= 4 * XPAD) {
     if constexpr (C::dev) return obs_step_tma<C>(P, B, phis, err, unit_rates, s);
-    else if (!P.obs_near) return cudaErrorInvalidValue;
-    else
+    else if (P.obs_near && P.pitch <= TILE_MAX_PITCH)
       return unit_rates ? launch_tile_kernel<C, MODEL_AC, MODE_STEP, true, true>(P, B, s)
                         : launch_tile_kernel<C, MODEL_AC, MODE_STEP, false, true>(P, B, s);
   }
@@ -441,6 +440,7 @@ long long adjoint_blocks(int nx, int ny) {
 template <typename T>
 cudaError_t launch_adjoint_step(const Phys<T>& P, const void* state, long long pop_bytes, const AdjBufs& A,
                                 double* gacc, bool hist_only, bool unit_rates, cudaStream_t s) {
+  unit_rates = unit_rates && P.pitch <= TILE_MAX_PITCH;
   const T* fin = static_cast<const T*>(state);
   const T* gin = reinterpret_cast<const T*>(static_cast<const unsigned char*>(state) + pop_bytes);
   const T* hist = reinterpret_cast<const T*>(static_cast<const unsigned char*>(state) + 2 * pop_bytes);
