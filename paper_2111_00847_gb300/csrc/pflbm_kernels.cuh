@@ -1596,20 +1596,14 @@ __global__ void __launch_bounds__(TILE_THREADS, (TileCfg<typename C::value_t, MO
   unsigned char* const hb = reinterpret_cast<unsigned char*>(B.hist + ix(P, 5, 0, x0, y0));
   if (inner) {
     const TileAddr<T> F(B.fin, P, x0, y0), G(B.gin, P, x0, y0);
-    // the halo ring, a warp's share at a time: R rows below and R above (columns
-    // [0, bw), bw <= 32), then R columns on either side of all bh + 2R rows
-    const int shares = 2 * R + (2 * R * (bh + 2 * R) + 31) / 32, warps = (nth + 31) >> 5;
-    auto place = [&](int k, int& cx, int& cy) {
-      cx = tid & 31;
-      if (k < 2 * R) {
-        cy = k < R ? k - R : bh + k - R;
-        return cx < bw;
-      }
-      const int q = (k - 2 * R) * 32 + cx;
-      cy = q / (2 * R) - R;
-      cx = q % (2 * R);
+    // the halo ring: R rows below and above (columns [0, bw)), and R columns on
+    // either side of all bh + 2R rows
+    const int cells = 2 * R * (bh + 2 * R);
+    auto ring_row = [&](int j) { return j < R ? j - R : bh + j - R; };
+    auto side_at = [&](int e, int& cx, int& cy) {
+      cy = e / (2 * R) - R;
+      cx = e % (2 * R);
       cx = cx < R ? cx - R : bw + cx - R;
-      return cy < bh + R;
     };
     auto load_gh = [&]() {
       G.pull(o9, g);
@@ -1620,26 +1614,59 @@ __global__ void __launch_bounds__(TILE_THREADS, (TileCfg<typename C::value_t, MO
       }
     };
     T v[9];
-    int k = tid >> 5, cx, cy;
     if constexpr (MODEL == MODEL_AC) {
-      // the first share's loads go out before the thread's own nodes', whose
-      // latency they share (4096^2 FP32: 522 us a step; after f's: 610)
-      const bool on = k < shares && place(k, cx, cy);
+      // rows by the threads of the tile's first rows, sides by its last threads.
+      // The first share's loads go out before the thread's own nodes', whose
+      // latency they share (4096^2 FP32: 525 us a step; after f's: 610).  16384^2:
+      // 8.32 ms; with the shares dealt by warps, as below, 8.46
+      int cx = tx, cy = 0;
+      bool on = true;
+      if (ty < 2 * R) {
+        cy = ring_row(ty);
+      } else {
+        on = nth - 1 - tid < cells;
+        side_at(nth - 1 - tid, cx, cy);
+      }
       if (on) F.pull(TileAddr<T>::node(cx, cy, P.pitch), v);
       F.pull(o9, f);
       load_gh();
       if (on) sp[(cy + R) * pw + cx + R] = sum9(v);
-      k += warps;
+      // what is left: flat tiles' other rows, the first rows' threads' and small
+      // blocks' side columns
+      for (int j = ty + bh; j < 2 * R; j += bh) {
+        F.pull(TileAddr<T>::node(tx, ring_row(j), P.pitch), v);
+        sp[(ring_row(j) + R) * pw + tx + R] = sum9(v);
+      }
+      for (int e = nth - 1 - tid + (ty < 2 * R ? 0 : nth); e < cells; e += nth) {
+        side_at(e, cx, cy);
+        F.pull(TileAddr<T>::node(cx, cy, P.pitch), v);
+        sp[(cy + R) * pw + cx + R] = sum9(v);
+      }
     } else {
-      // a ring two nodes wide wants the registers: its loads before g's
+      // a ring two nodes wide wants the registers: its loads, a warp's share at a
+      // time (columns of the rows first; bw <= 32), before g's
+      const int shares = 2 * R + (cells + 31) / 32, warps = (nth + 31) >> 5;
+      auto place = [&](int k, int& cx, int& cy) {
+        cx = tid & 31;
+        if (k < 2 * R) {
+          cy = k < R ? k - R : bh + k - R;
+          return cx < bw;
+        }
+        const int q = (k - 2 * R) * 32 + cx;
+        cy = q / (2 * R) - R;
+        cx = q % (2 * R);
+        cx = cx < R ? cx - R : bw + cx - R;
+        return cy < bh + R;
+      };
       F.pull(o9, f);
+      int cx, cy;
+      for (int k = tid >> 5; k < shares; k += warps) {
+        if (!place(k, cx, cy)) continue;
+        F.pull(TileAddr<T>::node(cx, cy, P.pitch), v);
+        sp[(cy + R) * pw + cx + R] = sum9(v);
+      }
+      load_gh();
     }
-    for (; k < shares; k += warps) {
-      if (!place(k, cx, cy)) continue;
-      F.pull(TileAddr<T>::node(cx, cy, P.pitch), v);
-      sp[(cy + R) * pw + cx + R] = sum9(v);
-    }
-    if constexpr (MODEL == MODEL_CH) load_gh();
     sp[(ty + R) * pw + tx + R] = sum9(f);
     __syncthreads();
   } else {
