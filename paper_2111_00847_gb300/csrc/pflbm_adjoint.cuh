@@ -893,21 +893,10 @@ __global__ void __launch_bounds__(TILE_THREADS, 2)
   T f[9], g[9], lfs[9], lgs[9], lhn[5], h3 = T(0), h4 = T(0);
   if (inner) {
     const TileAddr<T> F(fin, P, x0, y0), G(gin, P, x0, y0), A(lf, P, x0, y0), C(lg, P, x0, y0);
-    const int shares = 2 + (2 * (bh + 2) + 31) / 32, warps = (nth + 31) >> 5;
-    auto place = [&](int k, int& cx, int& cy) {
-      cx = tid & 31;
-      if (k < 2) {
-        cy = k == 0 ? -1 : bh;
-        return cx < bw;
-      }
-      const int q = (k - 2) * 32 + cx;
-      cy = q / 2 - 1;
-      cx = (q & 1) ? bw : -1;
-      return cy < bh + 1;
-    };
+    const RingDeal<1> ring(bw, bh, nth);
     T v[9];
-    int k = tid >> 5, cx, cy;
-    const bool on = k < shares && place(k, cx, cy);
+    int k = ring.first(tid), cx, cy;
+    const bool on = ring.is_share(k) && ring.place(k, tid, cx, cy);
     if (on) F.pull(TileAddr<T>::node(cx, cy, P.pitch), v);
     F.pull(o9, f);
     G.pull(o9, g);
@@ -927,8 +916,8 @@ __global__ void __launch_bounds__(TILE_THREADS, 2)
       h4 = *reinterpret_cast<const T*>(hb + 4 * pc + o5);
     }
     if (on) sp[(cy + 1) * pw + cx + 1] = sum9(v);
-    for (k += warps; k < shares; k += warps) {
-      if (!place(k, cx, cy)) continue;
+    for (k += ring.warps; ring.is_share(k); k += ring.warps) {
+      if (!ring.place(k, tid, cx, cy)) continue;
       F.pull(TileAddr<T>::node(cx, cy, P.pitch), v);
       sp[(cy + 1) * pw + cx + 1] = sum9(v);
     }

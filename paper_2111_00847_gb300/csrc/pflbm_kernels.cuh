@@ -45,6 +45,8 @@
 #include <climits>
 #include <type_traits>
 
+#include "pflbm_ring.h"
+
 namespace pflbm {
 
 enum { MODEL_AC = 0, MODEL_CH = 1 };
@@ -1645,23 +1647,11 @@ __global__ void __launch_bounds__(TILE_THREADS, (TileCfg<typename C::value_t, MO
     } else {
       // a ring two nodes wide wants the registers: its loads, a warp's share at a
       // time (columns of the rows first; bw <= 32), before g's
-      const int shares = 2 * R + (cells + 31) / 32, warps = (nth + 31) >> 5;
-      auto place = [&](int k, int& cx, int& cy) {
-        cx = tid & 31;
-        if (k < 2 * R) {
-          cy = k < R ? k - R : bh + k - R;
-          return cx < bw;
-        }
-        const int q = (k - 2 * R) * 32 + cx;
-        cy = q / (2 * R) - R;
-        cx = q % (2 * R);
-        cx = cx < R ? cx - R : bw + cx - R;
-        return cy < bh + R;
-      };
+      const RingDeal<R> ring(bw, bh, nth);
       F.pull(o9, f);
       int cx, cy;
-      for (int k = tid >> 5; k < shares; k += warps) {
-        if (!place(k, cx, cy)) continue;
+      for (int k = ring.first(tid); ring.is_share(k); k += ring.warps) {
+        if (!ring.place(k, tid, cx, cy)) continue;
         F.pull(TileAddr<T>::node(cx, cy, P.pitch), v);
         sp[(cy + R) * pw + cx + R] = sum9(v);
       }
