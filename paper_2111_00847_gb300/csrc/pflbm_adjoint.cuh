@@ -979,7 +979,9 @@ __global__ void __launch_bounds__(TILE_THREADS, 2)
       b += red[1][k];
     }
     double sx = double(a), sy = double(b);
-    const unsigned mask = __activemask();  // blocks of fewer than 32 threads
+    // the lanes that are here, known from the block's size: the loop above leaves them
+    // after different numbers of turns, and the shuffles bring them together again
+    const unsigned mask = nth >= 32 ? 0xffffffffu : (1u << nth) - 1u;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
       const double ox = __shfl_down_sync(mask, sx, o), oy = __shfl_down_sync(mask, sy, o);

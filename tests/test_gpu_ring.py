@@ -67,3 +67,21 @@ def test_adjoint_on_tiles_of_partial_warps(pk, nx, ny):
         out.append([t.detach().numpy() for t in (phi_n, phi0.grad, G.grad)])
     for a, b in zip(*out):
         assert np.abs(a - b).max() <= 1e-3 * np.abs(a).max()
+
+
+@pytest.mark.parametrize("nx,ny", [(3, 40), (7, 30), (29, 400)])
+def test_gravity_gradient_on_blocks_of_partial_warps(pk, nx, ny):
+    """dJ/dG sums over blocks of 30, 28 and 60 threads; the bar of the adjoint's other comparisons with autograd."""
+    from oracle.torch_ref import TorchScheme
+    from paper_2111_00847_gb300.adjoint import rollout
+
+    case = W.noisy_drop(nx, ny, walls="y", noise=0.01, gravity=(W.GRAV_RHO, 1e-5, -2e-5))
+    wts = torch.from_numpy(W.uniform_array(7, nx * ny).reshape(ny, nx) - 0.5)
+    grads = []
+    for run in (lambda phi, G: TorchScheme(case.params).run(phi, G, 8)[0], lambda phi, G: rollout(phi, G, case.params, 8, 3)):
+        phi0 = torch.tensor(case.phi, requires_grad=True)
+        G = torch.tensor([case.params.gx, case.params.gy], dtype=torch.float64, requires_grad=True)
+        (run(phi0, G) * wts).sum().backward()
+        grads.append((phi0.grad, G.grad))
+    for a, b in zip(*grads):
+        assert (a - b).abs().max() <= 1e-9 * a.abs().max()

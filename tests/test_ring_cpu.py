@@ -53,3 +53,10 @@ def lib(tmp_path_factory):
 def test_every_ring_cell_is_stored(lib, radius):
     bad = [(bw, bh) for bw in range(1, 33) for bh in range(1, 256 // bw + 1) if lib.ring_faults(radius, bw, bh)]
     assert not bad, f"{len(bad)} tiles, e.g. {bad[:8]}"
+
+
+def test_no_shuffle_mask_depends_on_convergence():
+    """A warp's lanes need not have met again after a loop of differing trip counts: shuffle masks come from sizes."""
+    for name in os.listdir(CSRC):
+        with open(os.path.join(CSRC, name)) as fh:
+            assert "__activemask" not in fh.read(), name
