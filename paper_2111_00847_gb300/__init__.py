@@ -16,6 +16,7 @@ from __future__ import annotations
 
 import ctypes as C
 import os
+import sys
 
 import numpy as np
 
@@ -147,12 +148,23 @@ class LbmError(RuntimeError):
         self.code = code
 
 
-def _dptr(a):
+def _dptr(a, device: bool = True):
+    """Address of an array argument: a float64 numpy array, or a contiguous
+    float64 tensor in host memory or (device) on the current device, the one a
+    handle's calls run on; its size is the caller's to get right.  The library
+    reads and writes plain doubles, so any other tensor is refused."""
     if a is None:
         return None
-    if isinstance(a, np.ndarray):
+    torch = sys.modules.get("torch")
+    if torch is None or not isinstance(a, torch.Tensor):
         return a.ctypes.data_as(C.POINTER(C.c_double))
-    return C.cast(a.data_ptr(), C.POINTER(C.c_double))  # a contiguous float64 tensor on the handle's device
+    if a.dtype != torch.float64 or a.layout != torch.strided or not a.is_contiguous() or a.is_neg():
+        raise ValueError(f"a contiguous float64 tensor is needed, got {a.dtype}, shape {tuple(a.shape)}, "
+                         f"{'strides ' + str(a.stride()) if a.layout == torch.strided else a.layout}")
+    if a.device.type != "cpu" and not (device and a.is_cuda and a.device.index == torch.cuda.current_device()):
+        raise ValueError(f"the tensor must lie in host memory{' or on the current device' if device else ''}, "
+                         f"it lies on {a.device}")
+    return C.cast(a.data_ptr(), C.POINTER(C.c_double))
 
 
 # ---- one-to-one wrappers of the C entry points ------------------------------
@@ -250,7 +262,7 @@ def lbm_adjoint_init(h, state0_ptr: int, out: np.ndarray):
 
 
 def lbm_adjoint_gravity(h, out: np.ndarray):
-    _check(load().lbm_adjoint_gravity(h, _dptr(out)), h)
+    _check(load().lbm_adjoint_gravity(h, _dptr(out, device=False)), h)
 
 
 def lbm_create_slab(params: LbmParams, y_lo: int, ny_own: int, stream: int = 0,
