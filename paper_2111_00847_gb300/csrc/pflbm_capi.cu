@@ -4,6 +4,8 @@
 // caller-supplied allocator), the per-run constants handed to the kernels,
 // and the sequencing of launches on the handle's stream.  Every step of the
 // method runs in the device kernels of pflbm_kernels.cuh.
+#include <cuda.h>
+
 #include <algorithm>
 #include <atomic>
 #include <cmath>
@@ -15,6 +17,7 @@
 #include <vector>
 
 #include "../../include/pflbm.h"
+#include "pflbm_copy.h"
 #include "pflbm_launch.h"
 
 using namespace pflbm;
@@ -1047,9 +1050,6 @@ static long long state_bytes(const lbm_handle* h) {
   return 2 * h->pop_bytes + 5LL * h->plane * (long long)h->esize;
 }
 
-// states up to this size are copied by one kernel
-static constexpr long long COPY_KERNEL_BYTES = 64LL << 20;
-
 static int ensure_adjoint(lbm_handle* h) {
   if (h->have_adj) return LBM_OK;
   const size_t pl = (size_t)h->plane * h->esize;
@@ -1135,25 +1135,47 @@ __global__ void __launch_bounds__(256) k_copy_state(uint4* __restrict__ a, uint4
   }
 }
 
+// Place of a snapshot buffer; false: the runtime or the driver does not know it.
+static bool buffer_place(const void* buf, BufferPlace* out) {
+  cudaPointerAttributes at;
+  if (cudaPointerGetAttributes(&at, buf) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  // (the driver's entry point through the runtime: the library links no libcuda)
+  using RangeFn = CUresult (*)(CUdeviceptr*, size_t*, CUdeviceptr);
+  static const RangeFn range_of = [] {
+    void* fn = nullptr;
+    cudaDriverEntryPointQueryResult st;
+    const cudaError_t e = cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &fn, 12000, cudaEnableDefault, &st);
+    if (e != cudaSuccess) cudaGetLastError();
+    return e == cudaSuccess && st == cudaDriverEntryPointSuccess ? reinterpret_cast<RangeFn>(fn) : nullptr;
+  }();
+  CUdeviceptr start = 0;
+  size_t bytes = 0;
+  if (!range_of || range_of(&start, &bytes, (CUdeviceptr)(uintptr_t)buf) != CUDA_SUCCESS) return false;
+  *out = {(uintptr_t)buf, at.type == cudaMemoryTypeDevice, at.device, (uintptr_t)start, (uint64_t)bytes};
+  return true;
+}
+
 // Copies the state to or from buf (device memory), on the handle's stream.
 static int copy_state(lbm_handle* h, void* buf, bool to_buf) {
   void* const part[3] = {h->pops[0][h->cur], h->pops[1][h->cur], h->hist};
   const long long n[3] = {h->pop_bytes, h->pop_bytes, 5LL * h->plane * (long long)h->esize};
-  unsigned char* p = static_cast<unsigned char*>(buf);
-  if (state_bytes(h) <= COPY_KERNEL_BYTES && (uintptr_t)buf % 16 == 0) {
-    // the kernel touches memory of this device only (parts are 16-byte
-    // multiples: the pitch is a multiple of 32 elements)
-    cudaPointerAttributes at;
-    if (cudaPointerGetAttributes(&at, buf) == cudaSuccess && at.type == cudaMemoryTypeDevice && at.device == h->device) {
-      const long long words = state_bytes(h) / 16;
-      const int blocks = (int)std::min<long long>((words + 255) / 256, 152 * 8);
-      k_copy_state<<<blocks, 256, 0, h->stream>>>((uint4*)part[0], (uint4*)part[1], (uint4*)part[2], (uint4*)buf,
-                                                  n[0] / 16, n[1] / 16, n[2] / 16, to_buf ? 1 : 0);
-      CUDA_TRY(h, cudaGetLastError());
-      return LBM_OK;
-    }
-    cudaGetLastError();
+  int current = -1;
+  BufferPlace at;
+  const uintptr_t parts = (uintptr_t)part[0] | (uintptr_t)part[1] | (uintptr_t)part[2];
+  if (state_bytes(h) <= COPY_KERNEL_BYTES && cudaGetDevice(&current) == cudaSuccess && buffer_place(buf, &at) &&
+      copy_by_kernel(at, parts, state_bytes(h), h->device, current)) {
+    // (the parts' sizes are 16-byte multiples: the pitch is a multiple of 32 elements)
+    const long long words = state_bytes(h) / 16;
+    const int blocks = (int)std::min<long long>((words + 255) / 256, 152 * 8);
+    k_copy_state<<<blocks, 256, 0, h->stream>>>((uint4*)part[0], (uint4*)part[1], (uint4*)part[2], (uint4*)buf,
+                                                n[0] / 16, n[1] / 16, n[2] / 16, to_buf ? 1 : 0);
+    CUDA_TRY(h, cudaGetLastError());
+    return LBM_OK;
   }
+  unsigned char* p = static_cast<unsigned char*>(buf);
   for (int k = 0; k < 3; p += n[k], ++k)
     CUDA_TRY(h, cudaMemcpyAsync(to_buf ? p : part[k], to_buf ? part[k] : p, n[k], cudaMemcpyDeviceToDevice, h->stream));
   return LBM_OK;
