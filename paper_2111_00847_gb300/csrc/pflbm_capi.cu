@@ -363,14 +363,13 @@ template <class C>
 static cudaError_t launch_mode(lbm_handle* h, int mode, const Phys<typename C::value_t>& P,
                                const Bufs<typename C::value_t>& B) {
   using T = typename C::value_t;
+  const bool moments = h->prm.n_delta > 0.0 && h->prm.n_delta < N_DELTA_DEFAULT;  // see launch_tile_moments
   if constexpr (!C::dev)
-    if (use_tile<C>(h))
-      return launch_tile<C>(h->prm.phase_model, mode, P, B, h->unit_rates,
-                            h->prm.n_delta > 0.0 && h->prm.n_delta < N_DELTA_DEFAULT, h->stream);
+    if (use_tile<C>(h)) return launch_tile<C>(h->prm.phase_model, mode, P, B, h->unit_rates, moments, h->stream);
   if (!h->dobs) return launch_march<C>(h->prm.phase_model, mode, P, B, h->stream);
   T* phis = (T*)h->obs_planes;
-  return launch_obs<C>(h->prm.phase_model, mode, P, B, phis, phis + h->plane, h->unit_rates, h->derr, h->use_tma,
-                       h->stream);
+  return launch_obs<C>(h->prm.phase_model, mode, P, B, phis, phis + h->plane, h->unit_rates, moments, h->derr,
+                       h->use_tma, h->stream);
 }
 
 template <class C>

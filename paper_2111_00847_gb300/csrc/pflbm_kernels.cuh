@@ -1108,11 +1108,12 @@ __device__ __forceinline__ T chem_pot_rows(const Phys<T>& P, const T* pm, const 
   return P.beta4 * (ph - P.phiA) * (ph - P.phiB) * (ph - P.phibar) - P.kappa * lap;
 }
 
-// The update of the arithmetic type, from nine stencil values in D2Q9 order.
-template <class C, int MODEL, int MODE, bool UR, class Sink, typename T = typename C::value_t>
+// The update of the arithmetic type (MOM: the moment form), from nine stencil values in D2Q9 order.
+template <class C, int MODEL, int MODE, bool UR, bool MOM = sizeof(typename C::value_t) == 4, class Sink,
+          typename T = typename C::value_t>
 __device__ __forceinline__ void node_update_nine(const Phys<T>& P, const Sink& out, const T phi9[9], const T mu9[9],
                                                  const T f[9], const T g[9], const T h[5], T u_in, T v_in, T p_in) {
-  if constexpr (sizeof(T) == 4) {
+  if constexpr (MOM) {
     node_update_moments<C, MODEL, MODE, UR>(P, out, phi9, mu9, f, g, h, u_in, v_in, p_in);
   } else {
     Row3<T> fr[3], mr[3];
@@ -1469,7 +1470,7 @@ struct TileSink {
 // none, over their fluid diagonal neighbours; zero at solid nodes no fluid node
 // reads), then the wall ghosts, all in shared memory, so that an obstacle costs
 // no pass and no plane of its own.  sp: [bh + 4][bw + 4].
-template <class C, bool UR, typename T = typename C::value_t>
+template <class C, bool UR, bool MOM, typename T = typename C::value_t>
 __device__ __forceinline__ void tile_near_obstacle(const Phys<T>& P, const Bufs<T>& B, T* sp, int x0, int y0, int w,
                                                    int hgt, int tx, int ty, int tid, int nth) {
   const int nx = P.nx, ny = P.ny, pw = blockDim.x + 4;
@@ -1549,7 +1550,7 @@ __device__ __forceinline__ void tile_near_obstacle(const Phys<T>& P, const Bufs<
   pull9_obs<C>(B.gin, P, 1, x, y, m, g);
 #pragma unroll
   for (int k = 0; k < 5; ++k) h[k] = B.hist[ix(P, 5, k, x, y)];
-  Stencil<C, MODEL_AC> st;
+  Stencil<C, MODEL_AC, MOM> st;
   const T* const q = sp + (ty + 2) * pw + tx + 2;
   st.phi_rows(q - pw, q, q + pw);
   st.template update<MODE_STEP, UR>(P, out, f, g, h, T(0), T(0), T(0));
@@ -1585,7 +1586,7 @@ __global__ void __launch_bounds__(TILE_THREADS, (TileCfg<typename C::value_t, MO
 
   if constexpr (OBS) {
     if (P.obs_near[blockIdx.y * gridDim.x + blockIdx.x]) {
-      tile_near_obstacle<C, UR>(P, B, sp, x0, y0, w, hgt, tx, ty, tid, nth);
+      tile_near_obstacle<C, UR, MOM>(P, B, sp, x0, y0, w, hgt, tx, ty, tid, nth);
       return;
     }
   }

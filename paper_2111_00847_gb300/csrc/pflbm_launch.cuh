@@ -121,7 +121,10 @@ static cudaError_t launch_tile_kernel(const Phys<typename C::value_t>& P, const 
 // moment form, operation for operation: the scheme amplifies rounding there (a
 // one-ulp change of phi grows to 3e-3 in 2000 steps at n_delta = 3e-3, to 1e-14
 // at the default 5e-3), so any other order of operations is another trajectory.
-// Narrow channels relax all moments (UR = false), as they always have.
+// With obstacles too (obs_ac).  Under 16 columns they relax all nine moments (UR =
+// false), as the register-pipelined kernel that served such grids does: the 4 x 256
+// channel at n_delta = 1e-5 amplifies rounding by up to 1e7 (node_update's form left
+// it 4.9e-9 from where this one does).
 template <class C>
 static cudaError_t launch_tile_moments(int mode, const Phys<typename C::value_t>& P,
                                        const Bufs<typename C::value_t>& B, bool unit_rates, cudaStream_t s) {
@@ -306,7 +309,7 @@ cudaError_t launch_obs_links(const Phys<T>& P, const unsigned char* solid, uint1
   return cudaGetLastError();
 }
 
-template <class C, int MODEL, int MODE, bool UR>
+template <class C, int MODEL, int MODE, bool UR, bool MOM>
 static cudaError_t obs_passes(const Phys<typename C::value_t>& P, const Bufs<typename C::value_t>& B,
                               typename C::value_t* phis, typename C::value_t* mus, cudaStream_t s) {
   using T = typename C::value_t;
@@ -317,21 +320,21 @@ static cudaError_t obs_passes(const Phys<typename C::value_t>& P, const Bufs<typ
     k_obs_mu<T><<<grid, OBS_THREADS, 0, s>>>(P, phis, mus, 0, P.nx, 0);
     if (fill_blocks) k_obs_fill<T><<<fill_blocks, OBS_THREADS, 0, s>>>(P, mus);
   }
-  k_obs_node<C, MODEL, MODE, UR><<<grid, OBS_THREADS, 0, s>>>(P, B, phis, mus);
+  k_obs_node<C, MODEL, MODE, UR, MOM><<<grid, OBS_THREADS, 0, s>>>(P, B, phis, mus);
   return cudaGetLastError();
 }
 
-template <class C, int MODEL>
+template <class C, int MODEL, bool MOM = sizeof(typename C::value_t) == 4>
 static cudaError_t obs_model(int mode, const Phys<typename C::value_t>& P, const Bufs<typename C::value_t>& B,
                              typename C::value_t* phis, typename C::value_t* mus, bool unit_rates,
                              cudaStream_t s) {
   switch (mode) {
     case MODE_STEP:
-      return unit_rates ? obs_passes<C, MODEL, MODE_STEP, true>(P, B, phis, mus, s)
-                        : obs_passes<C, MODEL, MODE_STEP, false>(P, B, phis, mus, s);
-    case MODE_MACRO: return obs_passes<C, MODEL, MODE_MACRO, false>(P, B, phis, mus, s);
-    case MODE_HIST: return obs_passes<C, MODEL, MODE_HIST, false>(P, B, phis, mus, s);
-    case MODE_INIT: return obs_passes<C, MODEL, MODE_INIT, false>(P, B, phis, mus, s);
+      return unit_rates ? obs_passes<C, MODEL, MODE_STEP, true, MOM>(P, B, phis, mus, s)
+                        : obs_passes<C, MODEL, MODE_STEP, false, MOM>(P, B, phis, mus, s);
+    case MODE_MACRO: return obs_passes<C, MODEL, MODE_MACRO, false, MOM>(P, B, phis, mus, s);
+    case MODE_HIST: return obs_passes<C, MODEL, MODE_HIST, false, MOM>(P, B, phis, mus, s);
+    case MODE_INIT: return obs_passes<C, MODEL, MODE_INIT, false, MOM>(P, B, phis, mus, s);
     default: return cudaErrorInvalidValue;
   }
 }
@@ -408,21 +411,34 @@ static cudaError_t obs_step_tma_ch(const Phys<typename C::value_t>& P0, const Bu
                     : launch_tma_ch_seg<C, false, true, true>(P, B, err, s, prev);
 }
 
-template <class C>
-cudaError_t launch_obs(int model, int mode, const Phys<typename C::value_t>& P, const Bufs<typename C::value_t>& B,
-                       typename C::value_t* phis, typename C::value_t* mus, bool unit_rates, int* err,
-                       bool use_tma, cudaStream_t s) {
-  if (!P.obs || !phis || (model == MODEL_CH && !mus)) return cudaErrorInvalidValue;
-  if (use_tma && model == MODEL_AC && mode == MODE_STEP && P.nx >= 4 * XPAD) {
+// Allen-Cahn with obstacles in the node update's form MOM.
+template <class C, bool MOM>
+static cudaError_t obs_ac(int mode, const Phys<typename C::value_t>& P, const Bufs<typename C::value_t>& B,
+                          typename C::value_t* phis, typename C::value_t* mus, bool unit_rates, int* err, bool use_tma,
+                          cudaStream_t s) {
+  if (use_tma && mode == MODE_STEP && P.nx >= 4 * XPAD) {
     if constexpr (C::dev) return obs_step_tma<C>(P, B, phis, err, unit_rates, s);
     else if (P.obs_near && P.pitch <= TILE_MAX_PITCH)
-      return unit_rates ? launch_tile_kernel<C, MODEL_AC, MODE_STEP, true, true>(P, B, s)
-                        : launch_tile_kernel<C, MODEL_AC, MODE_STEP, false, true>(P, B, s);
+      return unit_rates ? launch_tile_kernel<C, MODEL_AC, MODE_STEP, true, true, MOM>(P, B, s)
+                        : launch_tile_kernel<C, MODEL_AC, MODE_STEP, false, true, MOM>(P, B, s);
   }
-  if (use_tma && model == MODEL_CH && mode == MODE_STEP && P.nx >= 4 * XPAD)
-    return obs_step_tma_ch<C>(P, B, phis, mus, err, unit_rates, s);
-  return model == MODEL_CH ? obs_model<C, MODEL_CH>(mode, P, B, phis, mus, unit_rates, s)
-                           : obs_model<C, MODEL_AC>(mode, P, B, phis, mus, unit_rates, s);
+  return obs_model<C, MODEL_AC, MOM>(mode, P, B, phis, mus, unit_rates, s);
+}
+
+template <class C>
+cudaError_t launch_obs(int model, int mode, const Phys<typename C::value_t>& P, const Bufs<typename C::value_t>& B,
+                       typename C::value_t* phis, typename C::value_t* mus, bool unit_rates, bool moments, int* err,
+                       bool use_tma, cudaStream_t s) {
+  if (!P.obs || !phis || (model == MODEL_CH && !mus)) return cudaErrorInvalidValue;
+  if (model == MODEL_CH) {
+    if (use_tma && mode == MODE_STEP && P.nx >= 4 * XPAD)
+      return obs_step_tma_ch<C>(P, B, phis, mus, err, unit_rates, s);
+    return obs_model<C, MODEL_CH>(mode, P, B, phis, mus, unit_rates, s);
+  }
+  constexpr bool fp32 = sizeof(typename C::value_t) == 4;
+  if constexpr (!fp32)
+    if (moments) return obs_ac<C, true>(mode, P, B, phis, mus, unit_rates, err, use_tma, s);
+  return obs_ac<C, fp32>(mode, P, B, phis, mus, unit_rates, err, use_tma, s);
 }
 
 // Blocks of an adjoint node pass (each leaves a pair of dJ/dG partial sums).
@@ -507,7 +523,7 @@ cudaError_t launch_adjoint_init(const Phys<T>& P, const AdjBufs& A, double* out,
   template cudaError_t launch_march<C>(int, int, const Phys<C::value_t>&, const Bufs<C::value_t>&,  \
                                        cudaStream_t);                                               \
   template cudaError_t launch_obs<C>(int, int, const Phys<C::value_t>&, const Bufs<C::value_t>&,    \
-                                     C::value_t*, C::value_t*, bool, int*, bool, cudaStream_t);     \
+                                     C::value_t*, C::value_t*, bool, bool, int*, bool, cudaStream_t);     \
   template void obs_step_grid<C>(int, int, bool, int*, int*);
 
 #define PFLBM_INSTANTIATE_DEV(C)                                                                    \

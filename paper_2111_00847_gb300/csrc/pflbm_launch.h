@@ -60,13 +60,13 @@ cudaError_t launch_diag(const Phys<T>& P, const T* macro, const T* phi_prev, dou
 // from a dense byte mask, and one step (or MACRO / HIST / INIT pass) through
 // the obstacle passes; phis, mus: one-plane work planes of the arithmetic
 // type.  With use_tma the step runs on the tile (Allen-Cahn, plain storage) or
-// TMA kernels (err: their time-out flag).
+// TMA kernels (err: their time-out flag).  moments: as for launch_tile.
 template <typename T>
 cudaError_t launch_obs_links(const Phys<T>& P, const unsigned char* solid, uint16_t* obs, cudaStream_t s);
 template <class C>
 cudaError_t launch_obs(int model, int mode, const Phys<typename C::value_t>& P, const Bufs<typename C::value_t>& B,
-                       typename C::value_t* phis, typename C::value_t* mus, bool unit_rates, int* err,
-                       bool use_tma, cudaStream_t s);
+                       typename C::value_t* phis, typename C::value_t* mus, bool unit_rates, bool moments,
+                       int* err, bool use_tma, cudaStream_t s);
 // discrete adjoint of the Allen-Cahn step (pflbm_adjoint.cuh), plain storage
 template <typename T>
 cudaError_t launch_adjoint_step(const Phys<T>& P, const void* state, long long pop_bytes, const AdjBufs& A,

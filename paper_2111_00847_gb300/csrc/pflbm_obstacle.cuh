@@ -234,8 +234,8 @@ __global__ void k_obs_mu(const Phys<T> P, const T* __restrict__ phis, T* __restr
 // Node update of every node in a mode; solid nodes write zeros.  One node
 // per thread, so latency is hidden by residency alone: 8 blocks (32 warps)
 // per SM, 64 registers (measured 8.2 against 7.2 GLUPS at 6 blocks on the
-// 4096 x 2048 dam break over the obstacle, FP32).
-template <class C, int MODEL, int MODE, bool UR>
+// 4096 x 2048 dam break over the obstacle, FP32).  MOM: the update's moment form.
+template <class C, int MODEL, int MODE, bool UR, bool MOM>
 __global__ void __launch_bounds__(OBS_THREADS, 8) k_obs_node(const Phys<typename C::value_t> P,
                                                          const Bufs<typename C::value_t> B,
                                                          const typename C::value_t* __restrict__ phis,
@@ -285,7 +285,7 @@ __global__ void __launch_bounds__(OBS_THREADS, 8) k_obs_node(const Phys<typename
       for (int k = 0; k < 5; ++k) h[k] = B.hist[ix(P, 5, k, x, y)];
     }
   }
-  node_update_nine<C, MODEL, MODE, UR>(P, NodeSink<C, MODE>{P, B, x, y}, phi9, mu9, f, g, h, uin, vin, pin);
+  node_update_nine<C, MODEL, MODE, UR, MOM>(P, NodeSink<C, MODE>{P, B, x, y}, phi9, mu9, f, g, h, uin, vin, pin);
 }
 
 }  // namespace pflbm
