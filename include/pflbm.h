@@ -19,10 +19,11 @@
  *    [9][ny][nx] in the D2Q9 order c_0 = (0,0), c_1 = (1,0), c_2 = (0,1),
  *    c_3 = (-1,0), c_4 = (0,-1), c_5 = (1,1), c_6 = (-1,1), c_7 = (-1,-1),
  *    c_8 = (1,-1) (the order fixed by the matrix of Eq. (C.1)).  "Host"
- *    arrays of fields (lbm_init_fields, lbm_fields, lbm_set_fields,
- *    lbm_adjoint_seed, lbm_adjoint_init) may also lie in memory of the
- *    handle's device; a device array is read or written in order on the
- *    handle's stream, and lbm_adjoint_seed does not wait for that.
+ *    arrays of fields (lbm_init_fields, lbm_fields and its variants,
+ *    lbm_set_fields, lbm_adjoint_seed, lbm_adjoint_init) may also lie in
+ *    memory of the handle's device; a device array is read or written in
+ *    order on the handle's stream, and lbm_adjoint_seed does not wait for
+ *    that.
  *  - Boundaries: each side is periodic or a half-way bounce-back wall (no
  *    slip for g, no flux for f, Sec. 4) with the wetting condition of
  *    Eqs. (49)-(50) at the contact angle of that side.

@@ -571,6 +571,13 @@ static int do_fields(lbm_handle* h, int which, double* out, Region reg) {
     case LBM_DIAG: {
       int rc = run_diag<C>(h);
       if (rc) return rc;
+      cudaPointerAttributes at;
+      if (cudaPointerGetAttributes(&at, out) == cudaSuccess && at.type == cudaMemoryTypeDevice) {
+        CUDA_TRY(h, cudaMemcpyAsync(out, h->diag, sizeof(h->diag), cudaMemcpyHostToDevice, h->stream));
+        CUDA_TRY(h, cudaStreamSynchronize(h->stream));
+        return LBM_OK;
+      }
+      cudaGetLastError();
       std::memcpy(out, h->diag, sizeof(h->diag));
       return LBM_OK;
     }

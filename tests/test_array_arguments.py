@@ -96,3 +96,14 @@ def test_device_arrays_hold_what_host_arrays_hold(pk, prec):
                     pk.lbm_set_fields(s.handle, w, torch.tensor(host.fields(w), device="cuda"))
         for w in (pk.LBM_F_POP, pk.LBM_G_POP, pk.LBM_HIST):
             assert np.array_equal(s.fields(w), host.fields(w))
+
+
+@pytest.mark.gpu
+def test_diagnostics_into_a_device_array(pk):
+    case = W.noisy_drop(37, 29)
+    with pk.Simulation(case.params) as s:
+        s.init_fields(case.phi, case.ux, case.uy, case.p)
+        s.step(3)
+        out = torch.full((pk.LBM_NDIAG,), 7.0, dtype=torch.float64, device="cuda")
+        pk.lbm_fields(s.handle, pk.LBM_DIAG, out)
+        assert np.array_equal(out.cpu().numpy(), s.fields(pk.LBM_DIAG))
