@@ -639,11 +639,11 @@ __global__ void k_adj_reduce(const double* __restrict__ part, long long nparts, 
 // values in and 19 out, 4 and 1, 15 and 18 against 136 in all before.
 // In FP64 the pass is bound by the FP64 pipe: about 300 operations a node in
 // k_adj_tile, 640 in k_adj_node (512 x 2048: 1230 us in k_adj_node alone, 830 us
-// for all passes now; with 128 registers and 16 warps per SM, which spill 40
-// bytes, 8 % less time than with 150 and 8).  FP32 waits on memory: 500 x 1000
-// 110 us a step in all passes, 60 now.  Whole gradients, forward and
-// recomputation included: 512 x 2048 FP64 20 steps 47.7 -> 34.7 ms, 500 x 1000
-// FP32 40 steps 7.5 -> 6.2 ms.
+// for all passes now, 600 of them here; with 126 registers and 16 warps per SM,
+// 8 % less time than with 150 and 8).  FP32 waits on memory: 500 x 1000 110 us a
+// step in all passes, 60 now.  Whole gradients, forward and recomputation
+// included: 512 x 2048 FP64 20 steps 47.7 -> 34.5 ms, 500 x 1000 FP32 40 steps
+// 7.5 -> 5.7 ms (the last 0.4 and 0.5 ms by the fields' staying on the device).
 // ---------------------------------------------------------------------------
 constexpr int ADJ4 = 4;  // planes: phi, lap phi, d/dx, d/dy
 constexpr int ADJF = 2;  // f: moments 3, 5
@@ -812,61 +812,59 @@ __device__ __forceinline__ void node_adjoint_unit(const Phys<T>& P, const Row3<T
   o4[3] = lgy;
 }
 
-// Wetting ghosts of a phi tile (as in k_tile; after a barrier, ends with one where
-// there are any): the column beyond an x wall on every row the tile and its halo hold,
-// then the row beyond a y wall over the widened columns.  cl, cr, rb, rt: their
-// places relative to the tile (block-uniform; a Cahn-Hilliard tile that ends one
-// node short of a wall holds the ghosts too, for mu_phi of the node between).
-template <int R, typename T>
+// Wetting ghosts of a phi tile with a halo of one node (as in k_tile; after a
+// barrier, ends with one where there are any): the column beyond an x wall on every
+// row the tile and its halo hold, then the row beyond a y wall over the widened
+// columns (all block-uniform).
+template <typename T>
 __device__ __forceinline__ void tile_ghosts(const Phys<T>& P, T* sp, int pw, int x0, int y0, int w, int hgt, int tid,
                                             int nth) {
   const bool wx = P.wall_x != 0, wy = P.wall_y != 0;
-  const int cl = -1 - x0, cr = P.nx - x0, rb = -1 - y0, rt = P.ny - y0;
-  const bool has_l = wx && cl >= -R, has_r = wx && cr < w + R;
-  const bool has_b = wy && rb >= -R, has_t = wy && rt < hgt + R;
+  const bool has_l = wx && x0 == 0, has_r = wx && x0 + w == P.nx;
+  const bool has_b = wy && y0 == 0, has_t = wy && y0 + hgt == P.ny;
   if (has_l || has_r) {
-    for (int r = tid; r < hgt + 2 * R; r += nth) {
-      T* const q = sp + r * pw + R;
-      if (has_l) q[cl] = wall_ghost(P, SIDE_LEFT, q[cl + 1], q[cl + 2]);
-      if (has_r) q[cr] = wall_ghost(P, SIDE_RIGHT, q[cr - 1], q[cr - 2]);
+    for (int r = tid; r < hgt + 2; r += nth) {
+      T* const q = sp + r * pw + 1;
+      if (has_l) q[-1] = wall_ghost(P, SIDE_LEFT, q[0], q[1]);
+      if (has_r) q[w] = wall_ghost(P, SIDE_RIGHT, q[w - 1], q[w - 2]);
     }
     __syncthreads();
   }
   if (has_b || has_t) {
-    for (int c = tid; c < w + 2 * R; c += nth) {
-      T* const q = sp + R * pw + c;
-      if (has_b) q[rb * pw] = wall_ghost(P, SIDE_BOTTOM, q[(rb + 1) * pw], q[(rb + 2) * pw]);
-      if (has_t) q[rt * pw] = wall_ghost(P, SIDE_TOP, q[(rt - 1) * pw], q[(rt - 2) * pw]);
+    for (int c = tid; c < w + 2; c += nth) {
+      T* const q = sp + pw + c;
+      if (has_b) q[-pw] = wall_ghost(P, SIDE_BOTTOM, q[0], q[pw]);
+      if (has_t) q[hgt * pw] = wall_ghost(P, SIDE_TOP, q[(hgt - 1) * pw], q[(hgt - 2) * pw]);
     }
     __syncthreads();
   }
 }
 
-// phi of a tile's halo ring (in the domain, or wrapped), as k_tile forms it on
-// tiles at the grid's edge (written out there: as a call it cost the
-// Cahn-Hilliard step 100 bytes of spills, 4096^2 592 -> 670 us).
-template <class C, int MODE, int R, typename T = typename C::value_t>
-__device__ __forceinline__ void tile_ring(const Phys<T>& P, const Bufs<T>& B, T* sp, int pw, int x0, int y0, int w,
-                                          int hgt, int tid, int nth) {
+// phi of the halo ring, one node wide, of a tile at the grid's edge (in the domain,
+// or wrapped), as k_tile forms it there (written out there, for any ring: as a call
+// it cost the Cahn-Hilliard step 100 bytes of spills, 4096^2 592 -> 670 us).
+template <typename T>
+__device__ __forceinline__ void tile_ring(const Phys<T>& P, const T* fin, T* sp, int pw, int x0, int y0, int w, int hgt,
+                                          int tid, int nth) {
   const int nx = P.nx, ny = P.ny;
   const bool wx = P.wall_x != 0, wy = P.wall_y != 0;
-  const int row_cells = R * (w + 2 * R), ring = 2 * row_cells + 2 * R * hgt;
-  for (int k = tid; k < ring; k += nth) {
+  for (int k = tid; k < 2 * (w + 2 + hgt); k += nth) {
     int cx, cy;
-    if (k < 2 * row_cells) {
-      const int r = k / (w + 2 * R);
-      cx = k - r * (w + 2 * R) - R;
-      cy = r < R ? r - R : hgt + (r - R);
-    } else {
-      const int q = k - 2 * row_cells, r = q / (2 * R), c = q - r * 2 * R;
-      cy = r;
-      cx = c < R ? c - R : w + (c - R);
+    if (k < 2 * (w + 2)) {  // the rows below and above, over the widened columns
+      cy = k < w + 2 ? -1 : hgt;
+      cx = k - (k < w + 2 ? 0 : w + 2) - 1;
+    } else {  // the columns on either side
+      const int q = k - 2 * (w + 2);
+      cy = q >> 1;
+      cx = (q & 1) ? w : -1;
     }
     int xx = x0 + cx, yy = y0 + cy;
     if ((wx && (xx < 0 || xx >= nx)) || (wy && (yy < 0 || yy >= ny))) continue;  // ghosts follow
     xx = xx < 0 ? xx + nx : (xx >= nx ? xx - nx : xx);
     yy = yy < 0 ? yy + ny : (yy >= ny ? yy - ny : yy);
-    sp[(cy + R) * pw + cx + R] = phi_at<C, MODE>(P, B, xx, yy);
+    T v[9];
+    pull9<PopPlain<T>>(fin, P, 0, xx, yy, v);
+    sp[(cy + 1) * pw + cx + 1] = sum9(v);
   }
 }
 template <typename T>
@@ -935,9 +933,7 @@ __global__ void __launch_bounds__(TILE_THREADS, 2)
       for (int k = 0; k < 5; ++k) lhn[k] = lh[i5 + k * pc];
       if (!hist_only) h3 = hist[i5 + 3 * pc], h4 = hist[i5 + 4 * pc];
     }
-    Bufs<T> B;
-    B.fin = fin;
-    tile_ring<PopPlain<T>, MODE_STEP, 1>(P, B, sp, pw, x0, y0, w, hgt, tid, nth);
+    tile_ring(P, fin, sp, pw, x0, y0, w, hgt, tid, nth);
   }
   if (active) {
     const T ph = sum9(f);
@@ -947,7 +943,7 @@ __global__ void __launch_bounds__(TILE_THREADS, 2)
     if (!inner) phi[ix(P, 1, 0, x, y)] = ph;
   }
   __syncthreads();
-  if (!inner) tile_ghosts<1>(P, sp, pw, x0, y0, w, hgt, tid, nth);
+  if (!inner) tile_ghosts(P, sp, pw, x0, y0, w, hgt, tid, nth);
   T gxs = T(0), gys = T(0);
   if (active) {
     const T* const q = sp + (ty + 1) * pw + tx + 1;
