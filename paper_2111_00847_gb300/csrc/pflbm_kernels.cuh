@@ -446,8 +446,10 @@ __device__ __forceinline__ T wall_ghost(const Phys<T>& P, int side, T phi1, T ph
 // FP64 arithmetic of the node update.  GB300's FP64 pipe (two instructions a
 // clock and SM) bounds every FP64 kernel here, so operations are counted, and
 // each is written out with its own rounding (the compiler contracts nothing):
-// all kernels that update a node return the same bits, whichever of them the
-// size of a grid (or of a y-slab of it) selects.
+// node_update returns the same bits in every kernel that takes it (k_tile, k_obs_node,
+// k_step_tma_ch), whichever the size of a grid (or of a y-slab of it) selects.
+// k_march, and node_update_moments wherever it is asked for, round otherwise, and
+// the compiler contracts that form in each kernel by itself.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ double fm(double a, double b, double c) { return __fma_rn(a, b, c); }
 __device__ __forceinline__ double ad(double a, double b) { return __dadd_rn(a, b); }
@@ -1378,14 +1380,14 @@ __global__ void __launch_bounds__(BX) k_march(const Phys<typename C::value_t> P,
 // latency, and every SM gets nodes.  The ring is pulled again by the neighbouring
 // blocks, from L2 (DRAM moves 178 bytes per FP32 node update; the algorithmic
 // 184 less what L2 keeps).
-// What bounds it: FP32 by DRAM and its latency (4096^2: 522 us a step, 5.9 TB/s,
-// 0.87 of a copy); FP64 by the FP64 pipe (85 % busy, 209 instructions per node);
+// What bounds it: FP32 by DRAM and its latency (4096^2: 527 us a step, 5.9 TB/s,
+// 0.86 of a copy); FP64 by the FP64 pipe (85 % busy, 209 instructions per node);
 // small grids by one chain of launch, pull, barrier, update and store (4 us).
-// Measured, us a step, before -> now: FP32 128^2 20.4 -> 3.6, 300 x 150 21.8 ->
-// 4.7, 512^2 27.6 -> 9.7, 2048 x 1024 77.8 -> 70.3, 4096^2 558 -> 524, 8192^2
-// 2132 -> 2075, 16384^2 8324 -> 8259; FP64 4 x 256 857 -> 12, 128^2 103 -> 14.5,
-// 2048^2 2842 -> 1646 (with node_update); FP32 Cahn-Hilliard 128^2 23.9 -> 4.7,
-// 4096^2 717 -> 598.
+// Measured on one GPU in turn, us a step, before -> now: FP32 128^2 20.2 -> 3.7,
+// 300 x 150 21.6 -> 4.4, 512^2 27.9 -> 9.6, 2048 x 1024 78.6 -> 70.3, 4096^2 561
+// -> 527, 8192^2 2147 -> 2091, 16384^2 8337 -> 8318; FP64 4 x 256 854 -> 11.3 (16.2
+// in the moment form), 128^2 103 -> 14.3, 2048^2 2908 -> 1650 (with node_update);
+// FP32 Cahn-Hilliard 128^2 23.7 -> 6.2, 4096^2 726 -> 595.
 //
 // Interior tiles address everything from block-uniform bases with one 32-bit
 // offset per node (675 instructions per warp of nodes; 948 with per-node 64-bit

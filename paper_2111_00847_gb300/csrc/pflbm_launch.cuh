@@ -85,7 +85,7 @@ static cudaError_t launch_maybe_dependent(bool dependent, void (*kern)(KArgs...)
 }
 
 // Tile of the one-node-per-thread pass; columns in equal strips of at most 32.
-// FP32: 32 x 4 (4096^2: 522 us a step; 32 x 8 564); Cahn-Hilliard, whose ring is
+// FP32: 32 x 4 (4096^2: 522 us a step; 32 x 8 564, on one GPU); Cahn-Hilliard, whose ring is
 // two nodes wide: 32 x 8.  FP64: 32 x 8, and on grids of
 // few nodes 16 x 4 or 8 x 4, so that as many SMs as possible get nodes for
 // their FP64 pipes (300 x 150: 26.7 us; 32 x 8 33.1).
